@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(LSQ_THREADS, (EPL <= 16 ? 2 : 1)) fcg_step_ker
   if (cta == 0)
     for (int c = threadIdx.x; c < dp; c += blockDim.x) a.P[(int64_t)a.t * dp + c] = vec[c];
   if (MIXED) fused_pass_df<TA, EPL>(A, a.ld, d, dp, r0, r1, vec, wred, qred, a.part, P, cta);
-  else fused_pass<TA, EPL, (EPL <= 4)>(A, a.ld, d, dp, r0, r1, vec, wred, qred, a.part, P, cta);
+  else fused_pass<TA, EPL>(A, a.ld, d, dp, r0, r1, vec, wred, qred, a.part, P, cta);
   if (grid_barrier(a.bar, P, a.err)) return;
   // H p per column; q = <p, H p>, <p, r>
   double qp = 0.0, prp = 0.0;

@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(LSQ_THREADS, (EPL <= 16 ? 2 : 1)) solve_kernel
       fused_pass_df_staged<EPL>(reinterpret_cast<const double*>(A), a.ld, d, dp, r0, r1, vec, S.wred, S.qred, a.part,
                                 P, cta, slots);
     else if (MIXED) fused_pass_df<TA, EPL>(A, a.ld, d, dp, r0, r1, vec, S.wred, S.qred, a.part, P, cta);
-    else fused_pass<TA, EPL, (EPL <= 4)>(A, a.ld, d, dp, r0, r1, vec, S.wred, S.qred, a.part, P, cta);
+    else fused_pass<TA, EPL>(A, a.ld, d, dp, r0, r1, vec, S.wred, S.qred, a.part, P, cta);
   };
 
   // an FP32 pass: over the FP32 copy of A (COPY), else narrowing the rows of A as they arrive;
@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(LSQ_THREADS, (EPL <= 16 ? 2 : 1)) solve_kernel
       if (MIXED) {
         f32_pass(S.vec);
       } else {
-        fused_pass<TA, EPL, (!MIXED && EPL <= 4)>(A, a.ld, d, dp, r0, r1, S.vec, S.wred, S.qred, a.part, P, cta);
+        fused_pass<TA, EPL>(A, a.ld, d, dp, r0, r1, S.vec, S.wred, S.qred, a.part, P, cta);
         ++exact_passes;
       }
       ++passes;
