@@ -14,6 +14,7 @@
 
 #include "apass.cuh"
 #include "common.cuh"
+#include "fix96.cuh"
 
 namespace {
 
@@ -839,6 +840,195 @@ __global__ void __launch_bounds__(SRHT_THREADS, 1) srht_tma_kernel(
   }
 }
 
+// The FP64 transform of 2048-row blocks on the integer pipe (fix96.cuh).  In FP64 arithmetic the
+// transform is bound by the FP64 pipe: 11.5 additions an element took 17.6 of the 17.8 ms of the
+// sketch of 2^20 x 512 (m = 1024), where reading A takes 0.65 ms.  Here a CTA owns 4 columns
+// (32-byte row segments of FP64 A) and a range of blocks; per block each column gets the scale
+// of its largest element, the 11 butterfly levels run exactly on 96-bit integers (16 rows of a
+// column in registers per unit: bits 7..10 as the block is loaded, then bits 0..3 and 4..6 over
+// three word planes in shared memory), and only the sampled rows are rounded back to FP64 and
+// added to the CTA's partial of SA, which stays in registers (thread t owns sampled rows t,
+// t + 256, ...; more than 8 per thread in further grid.z slices, which transform the block
+// again).  4 columns keep the planes at 102 KB, so that two CTAs share an SM and one loads while
+// the other computes.  Columns with infinities or NaNs transform the signs of their infinities
+// instead: an output is +-inf where all of them agree, else NaN, as in floating point.
+// Measured (2^20 x 512 FP64, m = 1024, the whole sketch): 17.8 ms before, 4.36 ms; 144 instructions
+// an element, the integer pipe 55% busy, the rest waits on loads and shared memory.
+constexpr int SF_T = 256, SF_DC = 4, SF_LOGN2 = 11, SF_N2 = 1 << SF_LOGN2;
+constexpr int SF_PLANE = (SF_N2 + SF_N2 / 16) * SF_DC;  // words of a plane (zphys layout)
+constexpr size_t SF_SMEM = (size_t)3 * SF_PLANE * 4;
+
+__device__ __forceinline__ lsq_fix::i96 sf_load(const uint32_t* Z, int at) {
+  return lsq_fix::i96{Z[at], Z[SF_PLANE + at], Z[2 * SF_PLANE + at]};
+}
+__device__ __forceinline__ void sf_store(uint32_t* Z, int at, const lsq_fix::i96& v) {
+  Z[at] = v.w0;
+  Z[SF_PLANE + at] = v.w1;
+  Z[2 * SF_PLANE + at] = v.w2;
+}
+
+template <int K>
+__device__ __forceinline__ void sf_butterflies(lsq_fix::i96* v) {
+#pragma unroll
+  for (int h = 1; h < (1 << K); h <<= 1)
+#pragma unroll
+    for (int j = 0; j < (1 << K); ++j)
+      if (!(j & h)) {
+        const lsq_fix::i96 a = v[j], b = v[j + h];
+        v[j] = lsq_fix::add(a, b);
+        v[j + h] = lsq_fix::sub(a, b);
+      }
+}
+
+// levels over row bits [b, b + K) of the block in shared memory
+template <int K>
+__device__ __forceinline__ void sf_pass(uint32_t* Z, int b) {
+  for (int u = threadIdx.x; u < (SF_N2 >> K) * SF_DC; u += SF_T) {
+    const int c = u % SF_DC, q = u / SF_DC;
+    const int base = ((q >> b) << (b + K)) | (q & ((1 << b) - 1));
+    lsq_fix::i96 v[1 << K];
+#pragma unroll
+    for (int j = 0; j < (1 << K); ++j) v[j] = sf_load(Z, zphys(base + (j << b), SF_DC) + c);
+    sf_butterflies<K>(v);
+#pragma unroll
+    for (int j = 0; j < (1 << K); ++j) sf_store(Z, zphys(base + (j << b), SF_DC) + c, v[j]);
+  }
+}
+
+template <typename TA, int MY>
+__global__ void __launch_bounds__(SF_T, 2) srht_fix_kernel(const TA* __restrict__ A, int64_t n, int d, int64_t ld,
+                                                           int64_t N1, int64_t blocks_per_group,
+                                                           const uint32_t* __restrict__ signbits,
+                                                           const int64_t* __restrict__ rows_all, int m_all,
+                                                           double* __restrict__ part, uint32_t blk0) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  uint32_t* Z = reinterpret_cast<uint32_t*>(smem_raw);
+  // per column, by block parity: largest magnitude bits, number of infinities (NaN: above any)
+  __shared__ __align__(16) uint32_t mag_s[2][SF_DC];
+  __shared__ __align__(16) int ninf_s[2][SF_DC];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int c0 = blockIdx.x * SF_DC;
+  const int64_t gy = blockIdx.y;
+  const int64_t b_begin = gy * blocks_per_group, b_end = min(N1, b_begin + blocks_per_group);
+  const int s0 = (int)blockIdx.z * MY * SF_T;
+  const int m = min(m_all - s0, MY * SF_T);
+  uint32_t kk[MY];
+  double y[MY][SF_DC];
+#pragma unroll
+  for (int i = 0; i < MY; ++i) {
+    const int s = tid + SF_T * i;
+    kk[i] = s < m ? (uint32_t)rows_all[s0 + s] : 0u;
+#pragma unroll
+    for (int c = 0; c < SF_DC; ++c) y[i][c] = 0.0;
+  }
+  if (tid < 2 * SF_DC) {
+    (&mag_s[0][0])[tid] = 0u;
+    (&ninf_s[0][0])[tid] = 0;
+  }
+  // load units: column c of the tile, rows q + 128 j (j < 16); unit tid and unit tid + 256
+  const int c = tid % SF_DC, q = tid / SF_DC;
+  const bool col_ok = c0 + c < d;
+  constexpr int NAN_COUNT = 1 << 20;
+  __syncthreads();
+  for (int64_t i1 = b_begin; i1 < b_end; ++i1) {
+    const int par = (int)((i1 - b_begin) & 1);
+    const int64_t row0 = i1 << SF_LOGN2;
+    const int left = (int)min((int64_t)SF_N2, n - row0);  // rows of the block that exist
+    TA raw[2][16];
+    uint32_t mag = 0;
+    {
+      const TA* src = A + (row0 + q) * ld + c0 + c;
+      const int lq = col_ok ? left - q : 0;
+#pragma unroll
+      for (int j = 0; j < 16; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          raw[h][j] = 64 * h + 128 * j < lq ? __ldg(src) : (TA)0;
+          src += 64 * ld;
+        }
+      // the next block's 32-byte row segments on their way into L2 while this one is transformed
+      const TA* nxt = A + (row0 + SF_N2 + tid) * ld + c0;
+      const int64_t nleft = i1 + 1 < b_end ? n - row0 - SF_N2 - tid : 0;
+#pragma unroll
+      for (int j = 0; j < SF_N2 / SF_T; ++j) {
+        if (SF_T * j < nleft) asm volatile("prefetch.global.L2 [%0];" ::"l"(nxt));
+        nxt += SF_T * ld;
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int j = 0; j < 16; ++j) mag = max(mag, lsq_fix::mag_bits(raw[h][j]));
+#pragma unroll
+    for (int o = SF_DC; o < 32; o <<= 1) mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, o));
+    if (lane < SF_DC) atomicMax(&mag_s[par][c], mag);
+    __syncthreads();  // the scales are known, and the previous block's samples have been taken
+    const int emax = lsq_fix::scale_of<TA>(mag_s[par][c]);
+    if (tid < SF_DC) {
+      mag_s[par ^ 1][tid] = 0u;
+      ninf_s[par ^ 1][tid] = 0;
+    }
+    const uint32_t* sw = signbits + (row0 >> 5) + (q >> 5);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      lsq_fix::i96 v[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        const uint32_t flip = 0u - ((__ldg(sw + 2 * h + 4 * j) >> (q & 31)) & 1u);
+        v[j] = lsq_fix::to_fix(raw[h][j], emax, flip);
+        if (emax == lsq_fix::EXP_SPECIAL) {  // +-1 for infinities, 0 for finite values
+          const TA x = raw[h][j];
+          const bool nan = x != x, inf = !nan && lsq_fix::scale_of<TA>(lsq_fix::mag_bits(x)) == lsq_fix::EXP_SPECIAL;
+          v[j] = lsq_fix::negate_if(lsq_fix::i96{inf ? 1u : 0u, 0u, 0u}, flip ^ (x < (TA)0 ? ~0u : 0u));
+          if (nan || inf) atomicAdd(&ninf_s[par][c], nan ? NAN_COUNT : 1);
+        }
+      }
+      sf_butterflies<4>(v);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) sf_store(Z, zphys(q + 64 * h + 128 * j, SF_DC) + c, v[j]);
+    }
+    __syncthreads();
+    sf_pass<4>(Z, 0);
+    __syncthreads();
+    sf_pass<3>(Z, 4);
+    __syncthreads();
+    const uint32_t i1w = (uint32_t)i1 + blk0;  // the block's index in the whole (zero-padded) matrix
+    const uint4 mg = *reinterpret_cast<const uint4*>(mag_s[par]);
+    const int emv[SF_DC] = {lsq_fix::scale_of<TA>(mg.x), lsq_fix::scale_of<TA>(mg.y), lsq_fix::scale_of<TA>(mg.z),
+                            lsq_fix::scale_of<TA>(mg.w)};
+#pragma unroll
+    for (int i = 0; i < MY; ++i) {
+      if (tid + SF_T * i >= m) break;
+      const uint32_t flip = 0u - (uint32_t)(__popc((kk[i] >> SF_LOGN2) & i1w) & 1);
+      const int at = zphys((int)(kk[i] & (SF_N2 - 1)), SF_DC);
+      const uint4 z0 = *reinterpret_cast<const uint4*>(Z + at);
+      const uint4 z1 = *reinterpret_cast<const uint4*>(Z + SF_PLANE + at);
+      const uint4 z2 = *reinterpret_cast<const uint4*>(Z + 2 * SF_PLANE + at);
+      const lsq_fix::i96 zv[SF_DC] = {{z0.x, z1.x, z2.x}, {z0.y, z1.y, z2.y}, {z0.z, z1.z, z2.z}, {z0.w, z1.w, z2.w}};
+#pragma unroll
+      for (int k = 0; k < SF_DC; ++k) {
+        double add;
+        if (emv[k] != lsq_fix::EXP_SPECIAL) {
+          add = lsq_fix::from_fix(zv[k], emv[k], flip);
+        } else {
+          const int cnt = ninf_s[par][k], t = (int)lsq_fix::negate_if(zv[k], flip).w0;
+          add = t == cnt ? INFINITY : (t == -cnt ? -INFINITY : NAN);
+        }
+        y[i][k] += add;
+      }
+    }
+  }
+  double* out = part + (gy * m_all + s0) * d;
+#pragma unroll
+  for (int i = 0; i < MY; ++i) {
+    const int s = tid + SF_T * i;
+    if (s < m)
+#pragma unroll
+      for (int k = 0; k < SF_DC; ++k)
+        if (c0 + k < d) out[(int64_t)s * d + c0 + k] = y[i][k];
+  }
+}
+
 // ------------------------------------------------------------------------------------
 // SJLT: s distinct rows per column of S by Lemire's method on successive Philox words,
 // then a shared-memory scatter of each data row into its s target rows.
@@ -1173,6 +1363,51 @@ static bool srht_tma_launch(lsq_ctx* ctx, const lsq_matrix* A, int m, int64_t N1
   return true;
 }
 
+// the integer-pipe kernel of the FP64 transform (2048-row blocks)
+static int srht_fix_rows_per_thread(int m) {
+  const int my = lsq_ceil_div(m, SF_T);
+  return my <= 1 ? 1 : my <= 2 ? 2 : my <= 4 ? 4 : 8;
+}
+
+static lsq_status srht_fix_launch(lsq_ctx* ctx, const lsq_matrix* A, int m, int64_t N1, const uint32_t* signbits,
+                                  const int64_t* rows, double* part, int groups, int64_t blocks_per_group,
+                                  uint32_t blk0) {
+  const int d = (int)A->d, my = srht_fix_rows_per_thread(m);
+  const dim3 grid(lsq_ceil_div(d, SF_DC), groups, lsq_ceil_div(m, my * SF_T));
+  auto launch = [&](auto kern, auto* data) -> lsq_status {
+    LSQ_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SF_SMEM));
+    kern<<<grid, SF_T, SF_SMEM, ctx->stream>>>(data, A->n, d, A->ld, N1, blocks_per_group, signbits, rows, m, part,
+                                               blk0);
+    LSQ_LAUNCH_CHECK();
+    return LSQ_OK;
+  };
+  auto pick = [&](auto* data) -> lsq_status {
+    using TA = std::remove_const_t<std::remove_pointer_t<decltype(data)>>;
+    switch (my) {
+      case 1: return launch(srht_fix_kernel<TA, 1>, data);
+      case 2: return launch(srht_fix_kernel<TA, 2>, data);
+      case 4: return launch(srht_fix_kernel<TA, 4>, data);
+      default: return launch(srht_fix_kernel<TA, 8>, data);
+    }
+  };
+  return A->dtype == LSQ_F64 ? pick(static_cast<const double*>(A->data)) : pick(static_cast<const float*>(A->data));
+}
+
+// row-block groups whose CTAs (tiles of each group, `resident` at a time) finish soonest: whole
+// waves of equal groups, each group's partial sums costing about an eighth of a block
+static int64_t srht_pick_groups(int64_t tiles, int64_t resident, int64_t N1, int64_t cap) {
+  int64_t best = 1;
+  double best_cost = 1e300;
+  for (int64_t g = 1; g <= std::min<int64_t>(std::min(N1, cap), 64); ++g) {
+    const double cost = (double)((tiles * g + resident - 1) / resident) * ((double)((N1 + g - 1) / g) + 0.125);
+    if (cost < best_cost * (1.0 - 1e-9)) {
+      best_cost = cost;
+      best = g;
+    }
+  }
+  return best;
+}
+
 template <typename TC, int DC>
 static lsq_status srht_launch(lsq_ctx* ctx, const lsq_matrix* A, int m, int logN2, int64_t N1,
                               const uint32_t* signbits, const int64_t* rows, TC* part, int groups,
@@ -1274,6 +1509,13 @@ static lsq_status srht_run(lsq_ctx* ctx, const lsq_matrix* A, int m, uint64_t se
     while (logN2 > 0 && !fits(DC, logN2)) --logN2;
     if (!fits(DC, logN2) || logN2 > 16) return LSQ_ERR_ARG;
   }
+  // FP64 arithmetic on whole 2048-row blocks: the integer-pipe kernel, whose sampled partials are
+  // in registers (the general kernel stays for shorter transforms, zero-padded to N < 2048)
+  const bool fix = sizeof(TC) == 8 && logN >= SF_LOGN2;
+  if (fix) {
+    DC = SF_DC;
+    logN2 = SF_LOGN2;
+  }
   if (row0 % ((int64_t)1 << logN2) != 0) return LSQ_ERR_ARG;
   // blocks past the last row of A are all zero and add nothing
   const int64_t N1 = (A->n + ((int64_t)1 << logN2) - 1) >> logN2;
@@ -1284,6 +1526,9 @@ static lsq_status srht_run(lsq_ctx* ctx, const lsq_matrix* A, int m, uint64_t se
   groups = std::min(groups, N1);
   const int64_t cap = std::max<int64_t>(1, ((int64_t)256 << 20) / ((int64_t)m * d * (int64_t)sizeof(TC)));
   groups = std::min(groups, cap);
+  if (fix)
+    groups = srht_pick_groups((int64_t)tiles * lsq_ceil_div(m, srht_fix_rows_per_thread(m) * SF_T),
+                              2 * (int64_t)ctx->sm_count, N1, cap);
   const int64_t blocks_per_group = (N1 + groups - 1) / groups;
   groups = (N1 + blocks_per_group - 1) / blocks_per_group;
 
@@ -1362,6 +1607,12 @@ static lsq_status srht_run(lsq_ctx* ctx, const lsq_matrix* A, int m, uint64_t se
         if (lst != LSQ_OK) return lst;
       }
       staged = launched = true;
+    }
+  }
+  if constexpr (sizeof(TC) == 8) {
+    if (fix) {
+      st = srht_fix_launch(ctx, A, m, N1, sb, rows, part, (int)groups, blocks_per_group, blk0);
+      launched = true;
     }
   }
   if (!launched) switch (DC) {
