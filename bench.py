@@ -69,11 +69,11 @@ SOLVE_TRAFFIC = {
 }
 
 
-# The same for the batched ring pass (bpass_ring_kernel): one FP32 pass of iteration 0 over every
+# The same for the batched pass over FP32 A (btile_kernel): one FP32 pass of iteration 0 over every
 # problem of the 64-problem batch (ncu --metrics gpu__time_duration.sum,dram__bytes_read.sum,
-# dram__bytes_write.sum -k regex:bpass_ring -s 1 -c 1, python bench.py --batch 64 --steps 1
+# dram__bytes_write.sum -k regex:btile -s 1 -c 1, python bench.py --batch 64 --steps 1
 # --warmup 1 --no-cpu --no-e2e): reads of A plus the chunk partials written, over A's bytes.  The
-# exact passes stream A through the same ring.
+# exact passes stream A through the same stages.
 BATCH_TRAFFIC = {
     "sources_sha256": "24f75dc8026795c2dccf6d3c67aa4f6b483408194d47cf2c6680f9ac32380ad6",
     "ratio": (2664949504 + 27429888) / 2663123140,
@@ -84,7 +84,7 @@ def batch_sources_sha256() -> str:
     import hashlib
 
     h = hashlib.sha256()
-    for f in ("bring.cuh", "batch.cu", "common.cuh", "apass.cuh"):
+    for f in ("bmma.cuh", "btile.cuh", "batch.cu", "common.cuh", "apass.cuh"):
         with open(os.path.join(ROOT, "paper_1911_02675_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
@@ -758,7 +758,7 @@ def run_batch(args):
     pass_bytes = sum(b * it for b, (it, _) in zip(a_bytes, per))
     achieved = pass_bytes / (solve_ms * 1e-3) / 1e9
     statuses = sorted(set(st for _, st in per))
-    # DRAM bytes of the passes from the calibrated ratio (the ring pass: FP32 A, mixed precision)
+    # DRAM bytes of the passes from the calibrated ratio (FP32 A, mixed precision)
     batch_traffic = None
     if args.precision == "mixed" and batch_sources_sha256() == BATCH_TRAFFIC["sources_sha256"]:
         batch_traffic = BATCH_TRAFFIC["ratio"] * pass_bytes
@@ -804,7 +804,7 @@ def run_batch(args):
                        "A_GiB": sum(a_bytes) / 2 ** 30},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
                          "traffic": batch_traffic, "peak_kind": f"{peak_kind} (burst copy)",
-                         "kernel": "the batched iterations (bpass_ring_kernel for FP32 A: the passes, about 90 % of "
+                         "kernel": "the batched iterations (btile_kernel for FP32 A: the passes, about 90 % of "
                                    "the solve phase; A bytes over the whole solve phase's time)",
                          "algorithmic_bytes_per_launch": pass_bytes},
             "cpu_baseline": cpu, "e2e": e2e, "clocks": clk.summary(), "gpu_launches": launches}), flush=True)
