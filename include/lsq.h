@@ -233,12 +233,11 @@ LSQ_API lsq_status lsq_factor_qr(lsq_ctx* ctx, const double* SA, int64_t m, int6
                                  double* W, int32_t* perm, int64_t* rank_out);
 
 /* lsq_factor_ex: lsq_factor with the arithmetic of the Gram matrix chosen.
- *   gram_precision : LSQ_PREC_F64 (= lsq_factor) or LSQ_PREC_MIXED, which forms
- *                    H_S = (SA)^T (SA) in double-FP32 on the FP32 pipe: each entry of SA is
- *                    split into a 21-bit head and the FP32 rounding of the rest (about 45
- *                    significant bits), products are exact (TwoProduct by FMA) and sums are
- *                    (head, tail) pairs (TwoSum), a relative error near 1e-13 per entry,
- *                    far below what an FP32 sketch (LSQ_SKETCH_F32) already carries.  The
+ *   gram_precision : LSQ_PREC_F64 (= lsq_factor) or LSQ_PREC_MIXED.  Either way H_S is summed from
+ *                    exact products of 8-bit digits of SA (columns in fixed point on the scale of their
+ *                    largest element): 8 digits and 63 bits under LSQ_PREC_F64, nearer to H_S than FP64
+ *                    multiply-adds; 7 digits and an error near 2^-49 of the columns' norms under
+ *                    LSQ_PREC_MIXED, far below what an FP32 sketch (LSQ_SKETCH_F32) already carries.  The
  *                    Cholesky factor and the inverse stay FP64.
  * Other arguments, results and status as lsq_factor; LSQ_ERR_ARG for another precision. */
 LSQ_API lsq_status lsq_factor_ex(lsq_ctx* ctx, const double* SA, int64_t m, int64_t d, double* R, double* W,

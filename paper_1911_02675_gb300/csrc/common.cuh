@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "lsq.h"
 
 #define LSQ_WARPS 8
@@ -79,6 +81,18 @@ lsq_status lsq_sjlt_batched(lsq_ctx* ctx, int nprob, const lsq_matrix* A, const 
                             double* const* SA, int bf16);
 // a32[i * ld32 + c] = FP32 narrowing of A[i][c] (FP64 A), on the context's stream (solve.cu)
 lsq_status lsq_narrow_copy(lsq_ctx* ctx, const lsq_matrix* A, float* a32, int64_t ld32);
+
+// The Gram matrix of a sketch (gram.cu): tiles (a, b) of the upper triangle, row panels and splits,
+// digits per element; lsq_gram_run adds up part[split][dp][dp] (the tiles that meet the upper triangle)
+// from the device copy of `tiles`, mag (d words) and planes (plane_bytes).
+struct LsqGramPlan {
+  int dp, dq, ns, panel, splits, rows_per_split;
+  size_t plane_bytes;
+  std::vector<int2> tiles;
+};
+LsqGramPlan lsq_gram_plan(const lsq_ctx* ctx, int m, int d, bool mixed);
+lsq_status lsq_gram_run(lsq_ctx* ctx, const LsqGramPlan& p, const double* SA, int m, int d, const int2* d_tiles,
+                        uint32_t* mag, uint32_t* planes, double* part);
 
 // Factorisations of many sketches (batched solves): W_p = R_p^{-1} and W_p^T; status_out[p]
 // (host) = LSQ_OK or LSQ_ERR_RANK; the Gram matrices in double-FP32 when df_gram.

@@ -1,7 +1,7 @@
 // factor.cu -- H_S = (SA)^T (SA) = R^T R and W = R^{-1} (Section 1, PCG paragraph;
 // Section 6: a factorisation of H_S costs O(m d^2) and makes each solve with H_S O(d^2)).
 //
-// (1) Gram G = (SA)^T (SA) in FP64: split-K tiles over the upper triangle, fixed-order
+// (1) Gram G = (SA)^T (SA) (gram.cu): split-K tiles over the upper triangle, fixed-order
 //     reduction, padded to dp = 32 ceil(d/32) with an identity block.
 // (2) One cooperative kernel: right-looking blocked Cholesky with 32 x 32 blocks
 //     (diagonal block on one CTA, panel and trailing update as 32 x 8 tile tasks over
@@ -47,66 +47,6 @@ __device__ __forceinline__ float2 df_split(double v) {
   return make_float2(h, t);
 }
 
-// part[split][dp][dp] (upper tiles only) = sum over the split's rows of SA^T SA, in FP64 or,
-// with DF, in double-FP32
-template <bool DF>
-__global__ void __launch_bounds__(256) gram_kernel(const double* __restrict__ SA, int m, int d, int dp,
-                                                   int rows_per_split, const int2* __restrict__ tiles,
-                                                   double* __restrict__ part) {
-  using E = typename std::conditional<DF, float2, double>::type;
-  __shared__ E Xa[TK][TB];
-  __shared__ E Xb[TK][TB];
-  const int2 tl = tiles[blockIdx.x];
-  const int a0 = tl.x * TB, b0 = tl.y * TB;
-  const int r_begin = blockIdx.y * rows_per_split;
-  const int r_end = min(m, r_begin + rows_per_split);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double acc[4][4] = {};
-  float ah[4][4] = {}, al[4][4] = {};
-  for (int r0 = r_begin; r0 < r_end; r0 += TK) {
-    for (int e = threadIdx.x; e < TK * TB; e += 256) {
-      const int k = e / TB, c = e % TB;
-      const int r = r0 + k;
-      const double va = (r < r_end && a0 + c < d) ? SA[(int64_t)r * d + a0 + c] : 0.0;
-      const double vb = (r < r_end && b0 + c < d) ? SA[(int64_t)r * d + b0 + c] : 0.0;
-      if constexpr (DF) {
-        Xa[k][c] = df_split(va);
-        Xb[k][c] = df_split(vb);
-      } else {
-        Xa[k][c] = va;
-        Xb[k][c] = vb;
-      }
-    }
-    __syncthreads();
-    if constexpr (DF) {
-      df_gram_step(Xa, Xb, ty, tx, ah, al);
-    } else {
-#pragma unroll
-      for (int k = 0; k < TK; ++k) {
-        double x[4], y[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) x[i] = Xa[k][ty + 16 * i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) y[j] = Xb[k][tx + 16 * j];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = fma(x[i], y[j], acc[i][j]);
-      }
-    }
-    __syncthreads();
-  }
-  double* out = part + (int64_t)blockIdx.y * dp * dp;
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int a = a0 + ty + 16 * i, b = b0 + tx + 16 * j;
-      const double v = DF ? (double)ah[i][j] + (double)al[i][j] : acc[i][j];
-      if (a < dp && b < dp) out[(int64_t)a * dp + b] = v;
-    }
-}
-
 // G = sum of the splits on the upper tiles, mirrored; identity on the padded diagonal
 __global__ void gram_reduce_kernel(const double* __restrict__ part, int splits, int d, int dp, double* __restrict__ G) {
   const int64_t total = (int64_t)dp * dp;
@@ -116,11 +56,7 @@ __global__ void gram_reduce_kernel(const double* __restrict__ part, int splits, 
     if (a >= d || b >= d) {
       v = (a == b) ? 1.0 : 0.0;
     } else {
-      const int lo = min(a, b), hi = max(a, b);
-      // the tile holding (lo, hi) is an upper tile (tile row <= tile column)
-      const int64_t idx = (int64_t)lo * dp + hi;
-      const bool upper_tile = (lo / TB) <= (hi / TB);
-      const int64_t src = upper_tile ? idx : (int64_t)hi * dp + lo;
+      const int64_t src = (int64_t)min(a, b) * dp + max(a, b);
       v = 0.0;
       for (int g = 0; g < splits; ++g) v += part[(int64_t)g * dp * dp + src];
     }
@@ -478,16 +414,8 @@ extern "C" lsq_status lsq_factor_ex(lsq_ctx* ctx, const double* SA, int64_t m, i
   const int di = (int)d, mi = (int)m;
   const int nblk = (di + 31) / 32, dp = nblk * 32;
 
-  // Gram tiles (upper triangle of 64 x 64 tiles) and split-K
-  const int nt = (dp + TB - 1) / TB;
-  std::vector<int2> tiles;
-  for (int a = 0; a < nt; ++a)
-    for (int b = a; b < nt; ++b) tiles.push_back(make_int2(a, b));
-  int splits = std::max(1, (2 * ctx->sm_count + (int)tiles.size() - 1) / (int)tiles.size());
-  splits = std::min(splits, std::max(1, mi / 64));
-  splits = std::min(splits, std::max(1, (int)(((int64_t)128 << 20) / ((int64_t)dp * dp * 8))));
-  const int rows_per_split = ((mi + splits - 1) / splits + TK - 1) / TK * TK;
-  splits = (mi + rows_per_split - 1) / rows_per_split;
+  const LsqGramPlan gp = lsq_gram_plan(ctx, mi, di, gram_precision == LSQ_PREC_MIXED);
+  const int splits = gp.splits;
 
   // inverse tree levels, deepest first
   std::vector<std::vector<int4>> by_depth;
@@ -502,7 +430,8 @@ extern "C" lsq_status lsq_factor_ex(lsq_ctx* ctx, const double* SA, int64_t m, i
   const int nlevels = (int)level_start.size() - 1;
 
   const size_t mat = (size_t)dp * dp;
-  size_t need = lsq_align256((size_t)splits * mat * 8) + 4 * lsq_align256(mat * 8) + lsq_align256(tiles.size() * 8) +
+  size_t need = lsq_align256((size_t)splits * mat * 8) + 4 * lsq_align256(mat * 8) + lsq_align256(gp.tiles.size() * 8) +
+                lsq_align256((size_t)di * 4) + lsq_align256(gp.plane_bytes) +
                 lsq_align256(std::max<size_t>(1, nodes.size()) * 16) + lsq_align256(level_start.size() * 4) +
                 lsq_align256(64);
   lsq_status st = lsq_ensure_scratch(ctx, need);
@@ -513,14 +442,16 @@ extern "C" lsq_status lsq_factor_ex(lsq_ctx* ctx, const double* SA, int64_t m, i
   double* Rf = cv.take<double>(mat);
   double* Wf = cv.take<double>(mat);
   double* Tb = cv.take<double>(mat);
-  int2* d_tiles = cv.take<int2>(tiles.size());
+  int2* d_tiles = cv.take<int2>(gp.tiles.size());
+  uint32_t* mag = cv.take<uint32_t>(di);
+  uint32_t* planes = cv.take<uint32_t>(gp.plane_bytes / 4);
   int4* d_nodes = cv.take<int4>(std::max<size_t>(1, nodes.size()));
   int* d_levels = cv.take<int>(level_start.size());
   unsigned* bar = cv.take<unsigned>(16);
   int* err = reinterpret_cast<int*>(bar + 8);
   cudaStream_t s = ctx->stream;
 
-  LSQ_CUDA_TRY(cudaMemcpyAsync(d_tiles, tiles.data(), tiles.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
+  LSQ_CUDA_TRY(cudaMemcpyAsync(d_tiles, gp.tiles.data(), gp.tiles.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
   if (!nodes.empty())
     LSQ_CUDA_TRY(cudaMemcpyAsync(d_nodes, nodes.data(), nodes.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
   LSQ_CUDA_TRY(cudaMemcpyAsync(d_levels, level_start.data(), level_start.size() * sizeof(int), cudaMemcpyHostToDevice, s));
@@ -528,12 +459,8 @@ extern "C" lsq_status lsq_factor_ex(lsq_ctx* ctx, const double* SA, int64_t m, i
   LSQ_CUDA_TRY(cudaMemsetAsync(Rf, 0, mat * 8, s));
   LSQ_CUDA_TRY(cudaMemsetAsync(Wf, 0, mat * 8, s));
 
-  const dim3 ggrid((unsigned)tiles.size(), (unsigned)splits);
-  if (gram_precision == LSQ_PREC_MIXED)
-    gram_kernel<true><<<ggrid, 256, 0, s>>>(SA, mi, di, dp, rows_per_split, d_tiles, part);
-  else
-    gram_kernel<false><<<ggrid, 256, 0, s>>>(SA, mi, di, dp, rows_per_split, d_tiles, part);
-  LSQ_LAUNCH_CHECK();
+  st = lsq_gram_run(ctx, gp, SA, mi, di, d_tiles, mag, planes, part);
+  if (st != LSQ_OK) return st;
   gram_reduce_kernel<<<std::min(4 * ctx->sm_count, (int)((mat + 255) / 256)), 256, 0, s>>>(part, splits, di, dp, G);
   LSQ_LAUNCH_CHECK();
 

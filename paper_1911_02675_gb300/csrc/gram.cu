@@ -1,0 +1,259 @@
+// gram.cu -- the Gram matrix H_S = (SA)^T (SA) of a sketch (Section 1, PCG paragraph) on the tensor
+// cores, from exact products of 8-bit digits.
+//
+// The FP64 pipe does 1.75 multiply-adds a clock an SM, warp-level BF16 MMAs 1024.  Each column of SA is
+// written in fixed point on the scale of its largest element, as NS balanced base-256 digits
+// (|D| <= 128, exact in BF16):  SA[r][a] = sum_i D_i[r][a] 256^(7-i) 2^(e_a - 1084),  63 bits below the
+// largest element at NS = 8.  A product of two digits is at most 2^14, so the FP32 accumulators hold
+// the sum over 128 rows of every pair with the same i + j exactly (8 pairs x 128 x 2^14 = 2^24); pairs
+// with i + j >= NS are dropped (2^-57 of the columns' norms at NS = 8, 2^-49 at 7).  The sums are
+// folded into 64-bit integers every 128 rows, and one FP64 rounding per element follows: the result is
+// nearer to H_S than FP64 multiply-adds (NS = 8, LSQ_PREC_F64) and than double-FP32 ones (NS = 7,
+// LSQ_PREC_MIXED), with the columns' scale taken out, whatever the rows.
+//
+// Bound by the MMAs: NS (NS + 1) / 2 for each 16 x 8 x 16 product.  Measured (single launch times
+// before: FP64 or double-FP32 multiply-adds in tiles of 64 x 64): 4096 x 1024 mixed 1.10 -> 0.45 ms (the whole
+// factor 3.25 -> 2.69); 256 x 64 FP64 75 -> 12 us.
+#include <algorithm>
+
+#include "common.cuh"
+
+namespace {
+
+constexpr int GT = 256;                 // threads of the product kernel: 8 warps of 16 x 16 outputs
+constexpr int BA = 64, BB = 32;         // its tile of H_S
+constexpr int KC = 16;                  // rows of SA per stage
+constexpr int FOLD = 128;               // rows between folds
+constexpr int PA = BA + 8, PB = BB + 8;  // row pitches in shared memory (16-byte pieces of 8 rows: distinct banks)
+
+// largest magnitude of every column (high words): mag[c], zeroed before
+__global__ void __launch_bounds__(256) gram_max_kernel(const double* __restrict__ SA, int m, int d,
+                                                       uint32_t* __restrict__ mag) {
+  const int c = blockIdx.x * 32 + (threadIdx.x & 31);
+  const int w = threadIdx.x >> 5;
+  if (c >= d) return;
+  uint32_t v = 0;
+  const int step = 8 * gridDim.y;
+  for (int r = blockIdx.y * 8 + w; r < m; r += step) {
+    const double x = SA[(int64_t)r * d + c];
+    const uint32_t hi = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu;
+    v = max(v, hi);
+  }
+  atomicMax(mag + c, v);
+}
+
+// digits of rows [r0, r0 + rows) of SA (zeros from m on): plane i at out + i rows dq, row pitch dq; two
+// columns a thread
+template <int NS>
+__global__ void __launch_bounds__(256) gram_digits_kernel(const double* __restrict__ SA, int m, int d, int dq, int r0,
+                                                          int rows, const uint32_t* __restrict__ mag,
+                                                          uint32_t* __restrict__ out) {
+  const int half = dq / 2;
+  const int64_t plane = (int64_t)rows * half;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < plane; e += (int64_t)gridDim.x * blockDim.x) {
+    const int r = (int)(e / half), c = 2 * (int)(e - (int64_t)r * half);
+    unsigned long long U[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      U[h] = 0x8080808080808080ull;
+      if (r0 + r < m && c + h < d) {
+        const double x = SA[(int64_t)(r0 + r) * d + c + h];
+        const uint32_t hi = (uint32_t)__double2hiint(x);
+        const int ec = (int)((hi >> 20) & 0x7FFu), emax = max((int)(mag[c + h] >> 20), 1);
+        const unsigned long long M =
+            ((unsigned long long)((hi & 0xFFFFFu) | (ec ? 0x100000u : 0u)) << 32) | (uint32_t)__double2loint(x);
+        const int sh = emax - max(ec, 1) - 9;  // M 2^-sh below 2^62
+        const unsigned long long t = sh <= 0 ? M << -sh : sh < 64 ? M >> sh : 0ull;
+        U[h] += (hi >> 31) ? 0ull - t : t;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+      // digit + 128 is a byte; 2^23 + byte - (2^23 + 128) is the digit, exact in its upper 16 bits
+      const uint32_t b0 = (uint32_t)(U[0] >> (56 - 8 * i)) & 0xFFu, b1 = (uint32_t)(U[1] >> (56 - 8 * i)) & 0xFFu;
+      const float f0 = __uint_as_float(0x4B000000u | b0) - 8388736.f, f1 = __uint_as_float(0x4B000000u | b1) - 8388736.f;
+      out[i * plane + e] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
+    }
+  }
+}
+
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const void* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((unsigned)__cvta_generic_to_shared(p)));
+}
+
+__device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// part[split][a][b] (+)= the sum over the split's rows of the panel, for one tile of H_S that meets its
+// upper triangle; planes as gram_digits_kernel writes them (rows a multiple of KC)
+template <int NS>
+__global__ void __launch_bounds__(GT, 1) gram_mma_kernel(const uint16_t* __restrict__ planes, int rows, int dq, int dp,
+                                                         int rows_per_split, const int2* __restrict__ tiles,
+                                                         const uint32_t* __restrict__ mag, int d, int accumulate,
+                                                         double* __restrict__ part) {
+  extern __shared__ __align__(16) uint16_t sm[];  // two stages of [NS][KC][PA] and [NS][KC][PB]
+  constexpr int SA_E = NS * KC * PA, SB_E = NS * KC * PB, ST = SA_E + SB_E;
+  const int2 tl = tiles[blockIdx.x];
+  const int a0 = tl.x * BA, b0 = tl.y * BB;
+  const int k0 = blockIdx.y * rows_per_split, k1 = min(rows, k0 + rows_per_split);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int wa = (warp & 3) * 16, wb = (warp >> 2) * 16;
+  const int64_t plane = (int64_t)rows * dq;
+  auto load = [&](int k, int st) {
+    uint16_t* dst = sm + st * ST;
+    for (int e = tid; e < NS * KC * (BA + BB) / 8; e += GT) {
+      const int row = e / ((BA + BB) / 8), p = e - row * ((BA + BB) / 8);
+      const int i = row / KC, r = row - i * KC;
+      const bool isa = p < BA / 8;
+      const uint16_t* src = planes + i * plane + (int64_t)(k + r) * dq + (isa ? a0 + 8 * p : b0 + 8 * (p - BA / 8));
+      uint16_t* o = isa ? dst + row * PA + 8 * p : dst + SA_E + row * PB + 8 * (p - BA / 8);
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(o)), "l"(src)
+                   : "memory");
+    }
+  };
+  float acc[NS][2][4];
+  long long hi[2][4], lo[2][4];
+#pragma unroll
+  for (int w = 0; w < NS; ++w)
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+#pragma unroll
+      for (int x = 0; x < 4; ++x) acc[w][n][x] = 0.f;
+#pragma unroll
+  for (int n = 0; n < 2; ++n)
+#pragma unroll
+    for (int x = 0; x < 4; ++x) hi[n][x] = lo[n][x] = 0;
+  // hi: sums of i + j <= 3 on the scale of 3, lo: of 4 .. 7 on the scale of 7
+  auto fold = [&]() {
+#pragma unroll
+    for (int n = 0; n < 2; ++n)
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        long long h = 0, l = 0;
+#pragma unroll
+        for (int w = 0; w < 4; ++w) h = h * 256 + __float2int_rn(acc[w][n][x]);
+#pragma unroll
+        for (int w = 4; w < 8; ++w) l = l * 256 + (w < NS ? __float2int_rn(acc[w < NS ? w : 0][n][x]) : 0);
+        hi[n][x] += h;
+        lo[n][x] += l;
+#pragma unroll
+        for (int w = 0; w < NS; ++w) acc[w][n][x] = 0.f;
+      }
+  };
+  // ldmatrix rows of this lane: A tile (16 columns of H_S's row range as M, 16 rows of SA as K), both
+  // stored [k][column] and read transposed
+  const int lr = (lane & 7) + ((lane >> 4) & 1) * 8, lc = ((lane >> 3) & 1) * 8;    // A: matrices (m, k) 00 10 01 11
+  const int br = (lane & 7) + ((lane >> 3) & 1) * 8, bc = ((lane >> 4) & 1) * 8;    // B: (k, n) 00 10 01 11
+  if (k0 < k1) load(k0, 0);  // (a short last panel leaves splits empty)
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  int since = 0;
+  for (int k = k0, st = 0; k < k1; k += KC, st ^= 1) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    if (k + KC < k1) load(k + KC, st ^ 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const uint16_t* As = sm + st * ST + lr * PA + wa + lc;
+    const uint16_t* Bs = sm + st * ST + SA_E + br * PB + wb + bc;
+    uint32_t b[NS][4];
+#pragma unroll
+    for (int j = 0; j < NS; ++j) ldsm4t(b[j], Bs + j * KC * PB);
+#pragma unroll
+    for (int i = 0; i < NS; ++i) {
+      uint32_t a[4];
+      ldsm4t(a, As + i * KC * PA);
+#pragma unroll
+      for (int j = 0; j < NS; ++j)
+        if (i + j < NS) {
+          mma_bf16_16816(acc[i + j][0], a, b[j][0], b[j][1]);
+          mma_bf16_16816(acc[i + j][1], a, b[j][2], b[j][3]);
+        }
+    }
+    since += KC;
+    if (since == FOLD) {
+      fold();
+      since = 0;
+    }
+  }
+  fold();
+  // H_S[a][b] = (hi 2^32 + lo) 2^56 2^(e_a - 1084) 2^(e_b - 1084), NaN where a column is not finite
+  const int g = lane >> 2, t = lane & 3;
+  double* out = part + (int64_t)blockIdx.y * dp * dp;
+  auto scale = [&](int c) -> double {
+    if (c >= d) return 0.0;
+    const int e = (int)(mag[c] >> 20);
+    if (e == 0x7FF) return __longlong_as_double(0x7FF8000000000000ll);
+    const int x = max(e, 1) - 1084 + 28 + 1023;  // 2^(e - 1056), possibly subnormal
+    return x > 0 ? __longlong_as_double((long long)x << 52) : __longlong_as_double(1ll << (51 + x));
+  };
+#pragma unroll
+  for (int n = 0; n < 2; ++n)
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      const int a = a0 + wa + g + (x >> 1) * 8, bcol = b0 + wb + n * 8 + 2 * t + (x & 1);
+      if (a < dp && bcol < dp) {
+        const double v = fma((double)hi[n][x], 4294967296.0, (double)lo[n][x]) * scale(a) * scale(bcol);
+        double* o = out + (int64_t)a * dp + bcol;
+        *o = accumulate ? *o + v : v;
+      }
+    }
+}
+
+template <int NS>
+lsq_status run(lsq_ctx* ctx, const double* SA, int m, int d, int dp, int dq, int panel, int splits, int rows_per_split,
+               const int2* d_tiles, int ntiles, uint32_t* mag, uint32_t* planes, double* part) {
+  cudaStream_t s = ctx->stream;
+  constexpr size_t smem = (size_t)2 * (NS * KC * PA + NS * KC * PB) * 2;
+  LSQ_CUDA_TRY(cudaFuncSetAttribute(gram_mma_kernel<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  for (int r0 = 0; r0 < m; r0 += panel) {
+    const int rows = std::min(panel, (m - r0 + KC - 1) / KC * KC);
+    const int64_t pairs = (int64_t)rows * (dq / 2);
+    const int grid = (int)std::min<int64_t>((pairs + 255) / 256, 8 * (int64_t)ctx->sm_count);
+    gram_digits_kernel<NS><<<grid, 256, 0, s>>>(SA, m, d, dq, r0, rows, mag, planes);
+    LSQ_LAUNCH_CHECK();
+    gram_mma_kernel<NS><<<dim3((unsigned)ntiles, (unsigned)splits), GT, smem, s>>>(
+        reinterpret_cast<const uint16_t*>(planes), rows, dq, dp, rows_per_split, d_tiles, mag, d, r0 > 0 ? 1 : 0, part);
+    LSQ_LAUNCH_CHECK();
+  }
+  return LSQ_OK;
+}
+
+constexpr int64_t PANEL_BYTES = (int64_t)256 << 20;  // digit planes of a panel of rows at most
+
+}  // namespace
+
+LsqGramPlan lsq_gram_plan(const lsq_ctx* ctx, int m, int d, bool mixed) {
+  LsqGramPlan p;
+  p.dp = (d + 31) / 32 * 32;
+  p.dq = (d + BA - 1) / BA * BA;
+  for (int a = 0; a * BA < p.dp; ++a)
+    for (int b = 0; b * BB < p.dp; ++b)
+      if (b * BB + BB > a * BA) p.tiles.push_back(make_int2(a, b));
+  p.ns = mixed ? 7 : 8;
+  // panels of whole folds; the splits of a panel in whole stages, at least 64 rows, about two CTAs an SM
+  const int64_t cap = PANEL_BYTES / ((int64_t)p.ns * p.dq * 2) / FOLD * FOLD;
+  const int mk = (m + KC - 1) / KC * KC;
+  p.panel = (int)std::min<int64_t>(mk, std::max<int64_t>(FOLD, cap));
+  int splits = std::max(1, (2 * ctx->sm_count + (int)p.tiles.size() - 1) / (int)p.tiles.size());
+  splits = std::min(splits, std::max(1, p.panel / 64));
+  p.rows_per_split = ((p.panel + splits - 1) / splits + KC - 1) / KC * KC;
+  p.splits = (p.panel + p.rows_per_split - 1) / p.rows_per_split;
+  p.plane_bytes = (size_t)p.ns * p.panel * p.dq * 2;
+  return p;
+}
+
+lsq_status lsq_gram_run(lsq_ctx* ctx, const LsqGramPlan& p, const double* SA, int m, int d, const int2* d_tiles,
+                        uint32_t* mag, uint32_t* planes, double* part) {
+  LSQ_CUDA_TRY(cudaMemsetAsync(mag, 0, (size_t)d * 4, ctx->stream));
+  const int cb = (d + 31) / 32;
+  const int rb = std::max(1, std::min((m + 7) / 8, (4 * ctx->sm_count + cb - 1) / cb));
+  gram_max_kernel<<<dim3((unsigned)cb, (unsigned)rb), 256, 0, ctx->stream>>>(SA, m, d, mag);
+  LSQ_LAUNCH_CHECK();
+  const int nt = (int)p.tiles.size();
+  return p.ns == 8 ? run<8>(ctx, SA, m, d, p.dp, p.dq, p.panel, p.splits, p.rows_per_split, d_tiles, nt, mag, planes, part)
+                   : run<7>(ctx, SA, m, d, p.dp, p.dq, p.panel, p.splits, p.rows_per_split, d_tiles, nt, mag, planes, part);
+}
