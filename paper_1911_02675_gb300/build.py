@@ -14,7 +14,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "liblsq.so")
-SOURCES = ["ctx.cu", "sketch.cu", "sjlt.cu", "gauss_tc.cu", "factor.cu", "gram.cu", "solve.cu", "grad.cu", "advise.cu", "noalloc.cu", "fcg.cu",
+SOURCES = ["ctx.cu", "sketch.cu", "sjlt.cu", "gauss_tc.cu", "gauss64.cu", "factor.cu", "gram.cu", "solve.cu", "grad.cu", "advise.cu", "noalloc.cu", "fcg.cu",
            "batch.cu", "dist.cu", "qr.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

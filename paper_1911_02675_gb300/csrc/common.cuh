@@ -82,6 +82,14 @@ lsq_status lsq_sjlt_batched(lsq_ctx* ctx, int nprob, const lsq_matrix* A, const 
 // a32[i * ld32 + c] = FP32 narrowing of A[i][c] (FP64 A), on the context's stream (solve.cu)
 lsq_status lsq_narrow_copy(lsq_ctx* ctx, const lsq_matrix* A, float* a32, int64_t ld32);
 
+// The FP64 Gaussian sketch's partial sums (gauss64.cu)
+struct LsqGauss64 {
+  double* part;
+  int splits;
+};
+lsq_status lsq_gauss64_run(lsq_ctx* ctx, const lsq_matrix* A, int m, uint64_t seed, uint32_t t, int64_t grow0,
+                           LsqGauss64* out);
+
 // The Gram matrix of a sketch (gram.cu): tiles (a, b) of the upper triangle, row panels and splits,
 // digits per element; lsq_gram_run adds up part[split][dp][dp] (the tiles that meet the upper triangle)
 // from the device copy of `tiles`, mag (d words) and planes (plane_bytes).

@@ -1,0 +1,297 @@
+// gauss64.cu -- the Gaussian sketch SA = S A in FP64 (Section 2; the definition of lsq.h: Box-Muller on
+// 53-bit uniforms), its dense contraction from exact digit products (digits.cuh) on the tensor cores.
+//
+// FP64 multiply-adds run at 1.75 a clock an SM and the FP64 logarithm, square root, sine and cosine of a
+// pair of entries took ~100 FP64 instructions: 4096 x 64, m = 256, 219 us, where the 0.13 GFLOP and the
+// 2 MB of A are nothing.  Here a CTA owns a 64 x 64 tile of SA and a range of rows.  Per 16 rows it draws
+// its entries of S (table-driven log, sine and cosine with Taylor polynomials, a Goldschmidt square
+// root: ~40 FP64 instructions a pair), writes them as 8 base-256 digits in fixed point (2^-58) to shared
+// memory, and multiplies them with the digits of A's columns (columns in fixed point on the scale of their
+// largest element, digits_kernel): 36 digit products, each summed exactly in FP32 over 128 rows, then in
+// 64-bit integers.  S stays in shared memory.  The result is nearer to S A than FP64 multiply-adds.
+// Bound by the FP64 pipe (Box-Muller).  Measured (the sketch's kernels before its last
+// reduction): 4096 x 64, m = 256: 219 -> 77 us; m = 512: 381 -> 130 us.
+#include <math.h>
+
+#include <algorithm>
+
+#include "common.cuh"
+#include "digits.cuh"
+
+using namespace lsq_digits;
+
+namespace {
+
+constexpr int NS = 8;                // digits
+constexpr int T = 256;               // 8 warps, each 16 sketch rows x 32 columns of the tile
+constexpr int BM = 64, BN = 64, KC = 16, FOLD = 128;
+constexpr int PITCH = 64 + 8;        // row pitch in shared memory
+constexpr int OPER = NS * KC * PITCH;  // one operand's digits of a stage
+constexpr size_t SMEM = (size_t)4 * OPER * 2 + 128 * 16 + 64 * 16;
+
+struct Tables {
+  double2 lg[128];  // c ~ 1 / m of the interval, 2 ln c
+  double2 sc[64];   // sine and cosine at the middle of each 64th of a turn
+};
+
+// interval i of the mantissa [1, 2) in 128ths, the upper ones halved, so that the reduced argument lies
+// in [0.707, 1.414); c = 1 on both intervals that touch 1, which keeps ln near 1 accurate
+__device__ __forceinline__ bool upper(int i) { return i >= 53; }
+
+__device__ void fill_tables(Tables& tb) {
+  for (int i = threadIdx.x; i < 128; i += T) {
+    const double mid = (1.0 + (i + 0.5) / 128.0) * (upper(i) ? 0.5 : 1.0);
+    const double c = i == 0 || i == 127 ? 1.0 : 1.0 / mid;
+    tb.lg[i] = make_double2(c, 2.0 * log(c));
+  }
+  for (int i = threadIdx.x; i < 64; i += T) {
+    double s, c;
+    sincospi((i + 0.5) / 32.0, &s, &c);
+    tb.sc[i] = make_double2(s, c);
+  }
+}
+
+// z(2q, i) and z(2q + 1, i) from the words of Philox(i, q, t, TAG_GAUSS)
+__device__ __forceinline__ void normal_pair(const Tables& tb, uint4 w, double& zc, double& zs) {
+  const unsigned long long k1 = ((((unsigned long long)w.x << 32) | w.y) >> 11) * 2 + 1;  // u1 2^54
+  const unsigned long long k2 = ((((unsigned long long)w.z << 32) | w.w) >> 11) * 2 + 1;  // u2 2^54
+  // -2 ln u1: u1 = m 2^e, m c = 1 + r
+  const int lz = __clzll((long long)k1);
+  const unsigned long long n1 = k1 << lz;
+  const int i1 = (int)(n1 >> 56) & 127;
+  const bool up = upper(i1);
+  const double m = __longlong_as_double((long long)(((up ? 0x3FEull : 0x3FFull) << 52) | ((n1 >> 11) & 0xFFFFFFFFFFFFFull)));
+  const double2 lg = tb.lg[i1];
+  const double r = fma(m, lg.x, -1.0);
+  double p = fma(r, -2.0 / 7.0, 2.0 / 6.0);
+  p = fma(r, p, -2.0 / 5.0);
+  p = fma(r, p, 2.0 / 4.0);
+  p = fma(r, p, -2.0 / 3.0);
+  p = fma(r, p, 1.0);
+  p = fma(r * r, p, -2.0 * r);
+  const double x = fma((double)(lz - 9 - (up ? 1 : 0)), 2.0 * 0.69314718055994530942, lg.y + p);
+  // its square root: two Goldschmidt steps from the hardware's approximation, one correction
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  double g = x * y, h = 0.5 * y;
+  double e = fma(-g, h, 0.5);
+  g = fma(g, e, g);
+  h = fma(h, e, h);
+  e = fma(-g, h, 0.5);
+  g = fma(g, e, g);
+  const double rad = fma(fma(-g, g, x), h, g);
+  // sine and cosine of 2 pi u2 from the middle of its 64th of a turn
+  const double2 sc = tb.sc[(int)(k2 >> 48)];
+  const double a = (__longlong_as_double(0x4330000000000000ll | (long long)(k2 & 0xFFFFFFFFFFFFull)) - (0x1p52 + 0x1p47)) *
+                   (6.28318530717958647692 * 0x1p-54);
+  const double a2 = a * a;
+  double ps = fma(a2, -1.0 / 5040.0, 1.0 / 120.0);
+  ps = fma(a2, ps, -1.0 / 6.0);
+  const double sa = fma(a * a2, ps, a);
+  double pcs = fma(a2, 1.0 / 40320.0, -1.0 / 720.0);
+  pcs = fma(a2, pcs, 1.0 / 24.0);
+  pcs = fma(a2, pcs, -0.5);
+  const double cm = a2 * pcs;
+  zs = rad * (sc.x + fma(sc.x, cm, sc.y * sa));
+  zc = rad * (sc.y + fma(sc.y, cm, -(sc.x * sa)));
+}
+
+// part[split][j][c] (+)= sum over the split's rows of the panel of z(j, i) A[i][c]; planes: the digits of
+// the panel's rows (from row i0 of A, `rows` a multiple of KC)
+template <typename TA>
+__global__ void __launch_bounds__(T, 1) gauss64_kernel(const uint16_t* __restrict__ planes, int rows, int dq,
+                                                       const TA* __restrict__ A, int64_t n, int d, int64_t ld, int m,
+                                                       uint64_t seed, uint32_t t, int64_t i0, int64_t grow0,
+                                                       int rows_per_split, const uint32_t* __restrict__ mag,
+                                                       int accumulate, double* __restrict__ part) {
+  extern __shared__ __align__(16) uint16_t sm[];  // [2] digits of S, [2] digits of A, tables
+  Tables& tb = *reinterpret_cast<Tables*>(sm + 4 * OPER);
+  const int j0 = blockIdx.x * BM, c0 = blockIdx.y * BN;
+  const int k0 = blockIdx.z * rows_per_split, k1 = min(rows, k0 + rows_per_split);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int wa = (warp & 3) * 16, wb = (warp >> 2) * 32;
+  const int64_t plane = (int64_t)rows * dq;
+  auto load = [&](int k, int st) {
+    uint16_t* dst = sm + (2 + st) * OPER;
+    for (int e = tid; e < NS * KC * BN / 8; e += T) {
+      const int row = e / (BN / 8), p = e % (BN / 8), i = row / KC, r = row % KC;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                       (unsigned)__cvta_generic_to_shared(dst + row * PITCH + 8 * p)),
+                   "l"(planes + i * plane + (int64_t)(k + r) * dq + c0 + 8 * p)
+                   : "memory");
+    }
+  };
+  // 16 rows of S: row k + (tid mod 16), pairs tid / 16 and tid / 16 + 16
+  auto draw = [&](int k, int st) {
+    uint32_t* dst = reinterpret_cast<uint32_t*>(sm + st * OPER);
+    const int r = tid & 15;
+    const int64_t i = i0 + k + r;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int q = (tid >> 4) + 16 * h;
+      unsigned long long uc = BIAS, us = BIAS;
+      if (k + r < k1 && i < n) {
+        double zc, zs;
+        normal_pair(tb, philox_at(seed, (uint32_t)(i + grow0), (uint32_t)((j0 >> 1) + q), t, TAG_GAUSS), zc, zs);
+        uc = biased_digits(zc, 1026);  // 2^-58 units (|z| < 16)
+        us = biased_digits(zs, 1026);
+      }
+#pragma unroll
+      for (int x = 0; x < NS; ++x) dst[(x * KC + r) * (PITCH / 2) + q] = digit_pair(uc, us, x);
+    }
+  };
+  float acc[NS][4][4];
+  long long hi[4][4], lo[4][4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      hi[c][x] = lo[c][x] = 0;
+#pragma unroll
+      for (int w = 0; w < NS; ++w) acc[w][c][x] = 0.f;
+    }
+  auto fold = [&]() {
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        long long h = 0, l = 0;
+#pragma unroll
+        for (int w = 0; w < 4; ++w) h = h * 256 + __float2int_rn(acc[w][c][x]);
+#pragma unroll
+        for (int w = 4; w < 8; ++w) l = l * 256 + __float2int_rn(acc[w][c][x]);
+        hi[c][x] += h;
+        lo[c][x] += l;
+#pragma unroll
+        for (int w = 0; w < NS; ++w) acc[w][c][x] = 0.f;
+      }
+  };
+  const int lr = (lane & 7) + ((lane >> 4) & 1) * 8, lc = ((lane >> 3) & 1) * 8;
+  const int br = (lane & 7) + ((lane >> 3) & 1) * 8, bc = ((lane >> 4) & 1) * 8;
+  fill_tables(tb);
+  if (k0 < k1) load(k0, 0);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  __syncthreads();  // the tables are there
+  if (k0 < k1) draw(k0, 0);
+  int since = 0;
+  for (int k = k0, st = 0; k < k1; k += KC, st ^= 1) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();  // this stage is complete, and the other one no longer read
+    if (k + KC < k1) load(k + KC, st ^ 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const uint16_t* As = sm + st * OPER + lr * PITCH + wa + lc;
+    const uint16_t* Bs = sm + (2 + st) * OPER + br * PITCH + wb + bc;
+#pragma unroll
+    for (int j = 0; j < NS; ++j) {
+      uint32_t b0[4], b1[4];
+      ldsm4t(b0, Bs + j * KC * PITCH);
+      ldsm4t(b1, Bs + j * KC * PITCH + 16);
+#pragma unroll
+      for (int i = 0; i < NS; ++i)
+        if (i + j < NS) {
+          uint32_t a[4];
+          ldsm4t(a, As + i * KC * PITCH);
+          mma_bf16_16816(acc[i + j][0], a, b0[0], b0[1]);
+          mma_bf16_16816(acc[i + j][1], a, b0[2], b0[3]);
+          mma_bf16_16816(acc[i + j][2], a, b1[0], b1[1]);
+          mma_bf16_16816(acc[i + j][3], a, b1[2], b1[3]);
+        }
+    }
+    if (k + KC < k1) draw(k + KC, st ^ 1);
+    since += KC;
+    if (since == FOLD) {
+      fold();
+      since = 0;
+    }
+  }
+  fold();
+  // (hi 2^32 + lo) 2^56 2^-58 2^(emax - 1084); a column with infinities or NaNs: what its non-finite
+  // elements give in floating point
+  const int g = lane >> 2, tq = lane & 3;
+  double* out = part + (int64_t)blockIdx.z * m * d;
+#pragma unroll
+  for (int c = 0; c < 4; ++c)
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      const int j = j0 + wa + g + (x >> 1) * 8, col = c0 + wb + c * 8 + 2 * tq + (x & 1);
+      if (j < m && col < d) {
+        const int e = (int)(mag[col] >> 20);
+        double v = fma((double)hi[c][x], 4294967296.0, (double)lo[c][x]) * pow2(max(e, 1) - 1086);
+        if (e == 0x7FF) {
+          v = 0.0;
+          for (int k = k0; k < k1 && i0 + k < n; ++k) {
+            const double xa = (double)A[(i0 + k) * ld + col];
+            if (isfinite(xa)) continue;
+            double zc, zs;
+            normal_pair(tb, philox_at(seed, (uint32_t)(i0 + k + grow0), (uint32_t)(j >> 1), t, TAG_GAUSS), zc, zs);
+            v = fma((j & 1) ? zs : zc, xa, v);
+          }
+        }
+        double* o = out + (int64_t)j * d + col;
+        *o = accumulate ? *o + v : v;
+      }
+    }
+}
+
+constexpr int64_t PANEL_BYTES = (int64_t)256 << 20;  // digit planes of a panel of rows at most
+
+template <typename TA>
+lsq_status run(lsq_ctx* ctx, const lsq_matrix* A, int m, uint64_t seed, uint32_t t, int64_t grow0, LsqGauss64* out) {
+  const TA* data = static_cast<const TA*>(A->data);
+  const int d = (int)A->d, dq = (d + BN - 1) / BN * BN;
+  const int64_t n = A->n;
+  const int64_t cap = PANEL_BYTES / ((int64_t)NS * dq * 2) / FOLD * FOLD;
+  const int64_t panel = std::min<int64_t>((n + KC - 1) / KC * KC, std::max<int64_t>(FOLD, cap));
+  const int gx = lsq_ceil_div(m, BM), gy = dq / BN;
+  // whole waves of one CTA per SM; a CTA's start (tables, first stage) costs about a stage of rows
+  const int64_t stages = panel / KC;
+  const int64_t pcap = std::max<int64_t>(1, ((int64_t)256 << 20) / ((int64_t)m * d * 8));
+  int64_t splits = 1;
+  double best = 1e300;
+  for (int64_t s = 1; s <= std::min<int64_t>(std::min(stages, pcap), 1024); ++s) {
+    const double cost = (double)((gx * gy * s + ctx->sm_count - 1) / ctx->sm_count) * ((double)((stages + s - 1) / s) + 1.0);
+    if (cost < best * (1.0 - 1e-9)) {
+      best = cost;
+      splits = s;
+    }
+  }
+  const int rows_per_split = (int)((stages + splits - 1) / splits) * KC;
+  splits = (panel + rows_per_split - 1) / rows_per_split;
+  const size_t need = lsq_align256((size_t)splits * m * d * 8) + lsq_align256((size_t)NS * panel * dq * 2) +
+                      lsq_align256((size_t)d * 4);
+  lsq_status st = lsq_ensure_scratch(ctx, need);
+  if (st != LSQ_OK) return st;
+  Carver cv{reinterpret_cast<char*>(ctx->scratch), 0};
+  double* part = cv.take<double>((size_t)splits * m * d);
+  uint32_t* planes = cv.take<uint32_t>((size_t)NS * panel * dq / 2);
+  uint32_t* mag = cv.take<uint32_t>(d);
+  cudaStream_t s = ctx->stream;
+  LSQ_CUDA_TRY(cudaMemsetAsync(mag, 0, (size_t)d * 4, s));
+  const int cb = (d + 31) / 32;
+  const int rb = (int)std::max<int64_t>(1, std::min<int64_t>((n + 7) / 8, (4 * ctx->sm_count + cb - 1) / cb));
+  column_max_kernel<TA><<<dim3((unsigned)cb, (unsigned)rb), 256, 0, s>>>(data, n, d, A->ld, mag);
+  LSQ_LAUNCH_CHECK();
+  LSQ_CUDA_TRY(cudaFuncSetAttribute(gauss64_kernel<TA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM));
+  for (int64_t i0 = 0; i0 < n; i0 += panel) {
+    const int rows = (int)std::min<int64_t>(panel, (n - i0 + KC - 1) / KC * KC);
+    const int64_t pairs = (int64_t)rows * (dq / 2);
+    const int grid = (int)std::min<int64_t>((pairs + 255) / 256, 8 * (int64_t)ctx->sm_count);
+    digits_kernel<TA, NS><<<grid, 256, 0, s>>>(data, n, d, A->ld, dq, i0, rows, mag, planes);
+    LSQ_LAUNCH_CHECK();
+    gauss64_kernel<TA><<<dim3((unsigned)gx, (unsigned)gy, (unsigned)splits), T, SMEM, s>>>(
+        reinterpret_cast<const uint16_t*>(planes), rows, dq, data, n, d, A->ld, m, seed, t, i0, grow0, rows_per_split, mag,
+        i0 > 0 ? 1 : 0, part);
+    LSQ_LAUNCH_CHECK();
+  }
+  out->part = part;
+  out->splits = (int)splits;
+  return LSQ_OK;
+}
+
+}  // namespace
+
+// the partial sums [splits][m][d] of sqrt(m) SA, in the context's scratch
+lsq_status lsq_gauss64_run(lsq_ctx* ctx, const lsq_matrix* A, int m, uint64_t seed, uint32_t t, int64_t grow0,
+                           LsqGauss64* out) {
+  return A->dtype == LSQ_F64 ? run<double>(ctx, A, m, seed, t, grow0, out) : run<float>(ctx, A, m, seed, t, grow0, out);
+}

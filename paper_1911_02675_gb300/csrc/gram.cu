@@ -11,12 +11,15 @@
 // nearer to H_S than FP64 multiply-adds (NS = 8, LSQ_PREC_F64) and than double-FP32 ones (NS = 7,
 // LSQ_PREC_MIXED), with the columns' scale taken out, whatever the rows.
 //
-// Bound by the MMAs: NS (NS + 1) / 2 for each 16 x 8 x 16 product.  Measured (single launch times
-// before: FP64 or double-FP32 multiply-adds in tiles of 64 x 64): 4096 x 1024 mixed 1.10 -> 0.45 ms (the whole
-// factor 3.25 -> 2.69); 256 x 64 FP64 75 -> 12 us.
+// Bound by the MMAs, NS (NS + 1) / 2 for each 16 x 8 x 16 product, and the latency of a stage.  Measured
+// (maximum, digits and product; before: FP64 or double-FP32 multiply-adds in tiles of 64 x 64):
+// 4096 x 1024 mixed 1100 -> 568 us, 1204 x 301 FP64 169 -> 49 us, 256 x 64 FP64 75 -> 19 us.
 #include <algorithm>
 
 #include "common.cuh"
+#include "digits.cuh"
+
+using namespace lsq_digits;
 
 namespace {
 
@@ -26,71 +29,8 @@ constexpr int KC = 16;                  // rows of SA per stage
 constexpr int FOLD = 128;               // rows between folds
 constexpr int PA = BA + 8, PB = BB + 8;  // row pitches in shared memory (16-byte pieces of 8 rows: distinct banks)
 
-// largest magnitude of every column (high words): mag[c], zeroed before
-__global__ void __launch_bounds__(256) gram_max_kernel(const double* __restrict__ SA, int m, int d,
-                                                       uint32_t* __restrict__ mag) {
-  const int c = blockIdx.x * 32 + (threadIdx.x & 31);
-  const int w = threadIdx.x >> 5;
-  if (c >= d) return;
-  uint32_t v = 0;
-  const int step = 8 * gridDim.y;
-  for (int r = blockIdx.y * 8 + w; r < m; r += step) {
-    const double x = SA[(int64_t)r * d + c];
-    const uint32_t hi = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu;
-    v = max(v, hi);
-  }
-  atomicMax(mag + c, v);
-}
-
-// digits of rows [r0, r0 + rows) of SA (zeros from m on): plane i at out + i rows dq, row pitch dq; two
-// columns a thread
-template <int NS>
-__global__ void __launch_bounds__(256) gram_digits_kernel(const double* __restrict__ SA, int m, int d, int dq, int r0,
-                                                          int rows, const uint32_t* __restrict__ mag,
-                                                          uint32_t* __restrict__ out) {
-  const int half = dq / 2;
-  const int64_t plane = (int64_t)rows * half;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < plane; e += (int64_t)gridDim.x * blockDim.x) {
-    const int r = (int)(e / half), c = 2 * (int)(e - (int64_t)r * half);
-    unsigned long long U[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      U[h] = 0x8080808080808080ull;
-      if (r0 + r < m && c + h < d) {
-        const double x = SA[(int64_t)(r0 + r) * d + c + h];
-        const uint32_t hi = (uint32_t)__double2hiint(x);
-        const int ec = (int)((hi >> 20) & 0x7FFu), emax = max((int)(mag[c + h] >> 20), 1);
-        const unsigned long long M =
-            ((unsigned long long)((hi & 0xFFFFFu) | (ec ? 0x100000u : 0u)) << 32) | (uint32_t)__double2loint(x);
-        const int sh = emax - max(ec, 1) - 9;  // M 2^-sh below 2^62
-        const unsigned long long t = sh <= 0 ? M << -sh : sh < 64 ? M >> sh : 0ull;
-        U[h] += (hi >> 31) ? 0ull - t : t;
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < NS; ++i) {
-      // digit + 128 is a byte; 2^23 + byte - (2^23 + 128) is the digit, exact in its upper 16 bits
-      const uint32_t b0 = (uint32_t)(U[0] >> (56 - 8 * i)) & 0xFFu, b1 = (uint32_t)(U[1] >> (56 - 8 * i)) & 0xFFu;
-      const float f0 = __uint_as_float(0x4B000000u | b0) - 8388736.f, f1 = __uint_as_float(0x4B000000u | b1) - 8388736.f;
-      out[i * plane + e] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
-    }
-  }
-}
-
-__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const void* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"((unsigned)__cvta_generic_to_shared(p)));
-}
-
-__device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
 // part[split][a][b] (+)= the sum over the split's rows of the panel, for one tile of H_S that meets its
-// upper triangle; planes as gram_digits_kernel writes them (rows a multiple of KC)
+// upper triangle; planes as digits_kernel writes them (rows a multiple of KC)
 template <int NS>
 __global__ void __launch_bounds__(GT, 1) gram_mma_kernel(const uint16_t* __restrict__ planes, int rows, int dq, int dp,
                                                          int rows_per_split, const int2* __restrict__ tiles,
@@ -187,8 +127,7 @@ __global__ void __launch_bounds__(GT, 1) gram_mma_kernel(const uint16_t* __restr
     if (c >= d) return 0.0;
     const int e = (int)(mag[c] >> 20);
     if (e == 0x7FF) return __longlong_as_double(0x7FF8000000000000ll);
-    const int x = max(e, 1) - 1084 + 28 + 1023;  // 2^(e - 1056), possibly subnormal
-    return x > 0 ? __longlong_as_double((long long)x << 52) : __longlong_as_double(1ll << (51 + x));
+    return pow2(max(e, 1) - 1084 + 28);
   };
 #pragma unroll
   for (int n = 0; n < 2; ++n)
@@ -213,7 +152,7 @@ lsq_status run(lsq_ctx* ctx, const double* SA, int m, int d, int dp, int dq, int
     const int rows = std::min(panel, (m - r0 + KC - 1) / KC * KC);
     const int64_t pairs = (int64_t)rows * (dq / 2);
     const int grid = (int)std::min<int64_t>((pairs + 255) / 256, 8 * (int64_t)ctx->sm_count);
-    gram_digits_kernel<NS><<<grid, 256, 0, s>>>(SA, m, d, dq, r0, rows, mag, planes);
+    digits_kernel<double, NS><<<grid, 256, 0, s>>>(SA, m, d, d, dq, r0, rows, mag, planes);
     LSQ_LAUNCH_CHECK();
     gram_mma_kernel<NS><<<dim3((unsigned)ntiles, (unsigned)splits), GT, smem, s>>>(
         reinterpret_cast<const uint16_t*>(planes), rows, dq, dp, rows_per_split, d_tiles, mag, d, r0 > 0 ? 1 : 0, part);
@@ -251,7 +190,7 @@ lsq_status lsq_gram_run(lsq_ctx* ctx, const LsqGramPlan& p, const double* SA, in
   LSQ_CUDA_TRY(cudaMemsetAsync(mag, 0, (size_t)d * 4, ctx->stream));
   const int cb = (d + 31) / 32;
   const int rb = std::max(1, std::min((m + 7) / 8, (4 * ctx->sm_count + cb - 1) / cb));
-  gram_max_kernel<<<dim3((unsigned)cb, (unsigned)rb), 256, 0, ctx->stream>>>(SA, m, d, mag);
+  column_max_kernel<double><<<dim3((unsigned)cb, (unsigned)rb), 256, 0, ctx->stream>>>(SA, m, d, d, mag);
   LSQ_LAUNCH_CHECK();
   const int nt = (int)p.tiles.size();
   return p.ns == 8 ? run<8>(ctx, SA, m, d, p.dp, p.dq, p.panel, p.splits, p.rows_per_split, d_tiles, nt, mag, planes, part)

@@ -47,24 +47,9 @@ __device__ __forceinline__ double unit_open53(uint32_t hi, uint32_t lo) {
   return ((double)k + 0.5) * 0x1p-53;
 }
 
-// Box-Muller pair (cosine branch, sine branch) in the arithmetic type T
-template <typename T>
-__device__ __forceinline__ void box_muller(uint4 w, T& z_cos, T& z_sin);
-
-template <>
-__device__ __forceinline__ void box_muller<double>(uint4 w, double& zc, double& zs) {
-  const double u1 = unit_open53(w.x, w.y);
-  const double u2 = unit_open53(w.z, w.w);
-  const double rad = sqrt(-2.0 * log(u1));
-  double s, c;
-  sincospi(2.0 * u2, &s, &c);
-  zc = rad * c;
-  zs = rad * s;
-}
-
-template <>
-__device__ __forceinline__ void box_muller<float>(uint4 w, float& zc, float& zs) {
-  // the same 53-bit uniforms, evaluated in FP32 (u1 > 0 is kept by the +1/2 offset)
+// Box-Muller pair (cosine branch, sine branch): the 53-bit uniforms, evaluated in FP32 (u1 > 0 is kept
+// by the +1/2 offset)
+__device__ __forceinline__ void box_muller(uint4 w, float& zc, float& zs) {
   const float u1 = (float)unit_open53(w.x, w.y);
   const float u2 = (float)unit_open53(w.z, w.w);
   const float rad = sqrtf(-2.0f * logf(u1));
@@ -94,49 +79,49 @@ __global__ void reduce_splits_kernel(const TP* __restrict__ part, int splits, in
 }
 
 // ------------------------------------------------------------------------------------
-// Gaussian: SA = S A, S[j,i] = z(j,i)/sqrt(m).  Split-K GEMM over the rows of A; each
+// Gaussian in FP32 arithmetic: SA = S A, S[j,i] = z(j,i)/sqrt(m) (FP64: gauss64.cu; BF16: gauss_tc.cu).
+// Split-K GEMM over the rows of A; each
 // CTA owns a 64 x 64 tile of SA and a contiguous range of rows, regenerates its 64 x 16
 // tile of S per step (one Philox call per pair of sketch rows) and accumulates 4 x 4
 // outputs per thread.  Scaling by 1/sqrt(m) happens in the reduction.
 // ------------------------------------------------------------------------------------
 constexpr int GM = 64, GD = 64, GK = 16;
 
-template <typename T>
 __global__ void __launch_bounds__(256) gauss_sketch_kernel(const void* __restrict__ A, int dtype, int64_t n, int d,
                                                           int64_t ld, int m, uint64_t seed, uint32_t t,
-                                                          int64_t rows_per_split, T* __restrict__ part,
+                                                          int64_t rows_per_split, float* __restrict__ part,
                                                           int64_t grow0) {
-  __shared__ T Ss[GK][GM];
-  __shared__ T As[GK][GD];
+  __shared__ float Ss[GK][GM];
+  __shared__ float As[GK][GD];
   const int j0 = blockIdx.x * GM, c0 = blockIdx.y * GD;
   const int64_t i_begin = (int64_t)blockIdx.z * rows_per_split;
   const int64_t i_end = min(n, i_begin + rows_per_split);
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  T acc[4][4];
+  float acc[4][4];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = (T)0;
+    for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
 
   for (int64_t i0 = i_begin; i0 < i_end; i0 += GK) {
     for (int e = threadIdx.x; e < (GM / 2) * GK; e += 256) {
       const int jp = e / GK, k = e % GK;
       const int64_t i = i0 + k;
-      T zc = (T)0, zs = (T)0;
+      float zc = 0.f, zs = 0.f;
       if (i < i_end)
-        box_muller<T>(philox_at(seed, (uint32_t)(i + grow0), (uint32_t)((j0 >> 1) + jp), t, TAG_GAUSS), zc, zs);
+        box_muller(philox_at(seed, (uint32_t)(i + grow0), (uint32_t)((j0 >> 1) + jp), t, TAG_GAUSS), zc, zs);
       Ss[k][2 * jp] = zc;
       Ss[k][2 * jp + 1] = zs;
     }
     for (int e = threadIdx.x; e < GK * GD; e += 256) {
       const int k = e / GD, c = e % GD;
       const int64_t i = i0 + k;
-      As[k][c] = (i < i_end && c0 + c < d) ? load_as<T>(A, i * ld + c0 + c, dtype) : (T)0;
+      As[k][c] = (i < i_end && c0 + c < d) ? load_as<float>(A, i * ld + c0 + c, dtype) : 0.f;
     }
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < GK; ++k) {
-      T s[4], a[4];
+      float s[4], a[4];
 #pragma unroll
       for (int r = 0; r < 4; ++r) s[r] = Ss[k][ty + 16 * r];
 #pragma unroll
@@ -144,11 +129,11 @@ __global__ void __launch_bounds__(256) gauss_sketch_kernel(const void* __restric
 #pragma unroll
       for (int r = 0; r < 4; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = fma(s[r], a[c], acc[r][c]);
+        for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(s[r], a[c], acc[r][c]);
     }
     __syncthreads();
   }
-  T* out = part + (int64_t)blockIdx.z * m * d;
+  float* out = part + (int64_t)blockIdx.z * m * d;
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     const int j = j0 + ty + 16 * r;
@@ -1136,27 +1121,40 @@ static lsq_status validate_matrix(const lsq_matrix* A) {
   return LSQ_OK;
 }
 
-template <typename TC>
+// FP32 arithmetic
 static lsq_status gauss_run(lsq_ctx* ctx, const lsq_matrix* A, int m, uint64_t seed, uint32_t t, double* SA,
                             int64_t grow0) {
   const int d = (int)A->d;
   const int gx = lsq_ceil_div(m, GM), gy = lsq_ceil_div(d, GD);
   const int64_t ksteps = (A->n + GK - 1) / GK;
   int64_t splits = ((int64_t)2 * ctx->sm_count + gx * gy - 1) / (gx * gy);
-  const int64_t cap = std::max<int64_t>(1, ((int64_t)256 << 20) / ((int64_t)m * d * (int64_t)sizeof(TC)));
+  const int64_t cap = std::max<int64_t>(1, ((int64_t)256 << 20) / ((int64_t)m * d * (int64_t)sizeof(float)));
   splits = std::max<int64_t>(1, std::min(std::min(splits, ksteps), cap));
   const int64_t rows_per_split = ((ksteps + splits - 1) / splits) * GK;
   splits = (A->n + rows_per_split - 1) / rows_per_split;
-  lsq_status st = lsq_ensure_scratch(ctx, lsq_align256((size_t)splits * m * d * sizeof(TC)));
+  lsq_status st = lsq_ensure_scratch(ctx, lsq_align256((size_t)splits * m * d * sizeof(float)));
   if (st != LSQ_OK) return st;
-  TC* part = reinterpret_cast<TC*>(ctx->scratch);
+  float* part = reinterpret_cast<float*>(ctx->scratch);
   dim3 grid(gx, gy, (unsigned)splits);
-  gauss_sketch_kernel<TC><<<grid, 256, 0, ctx->stream>>>(A->data, A->dtype, A->n, d, A->ld, m, seed, t,
+  gauss_sketch_kernel<<<grid, 256, 0, ctx->stream>>>(A->data, A->dtype, A->n, d, A->ld, m, seed, t,
                                                           rows_per_split, part, grow0);
   LSQ_LAUNCH_CHECK();
   const int64_t md = (int64_t)m * d;
-  reduce_splits_kernel<TC><<<grid_for(md, 256, 4 * ctx->sm_count), 256, 0, ctx->stream>>>(
+  reduce_splits_kernel<float><<<grid_for(md, 256, 4 * ctx->sm_count), 256, 0, ctx->stream>>>(
       part, (int)splits, md, 1.0 / sqrt((double)m), SA);
+  LSQ_LAUNCH_CHECK();
+  return LSQ_OK;
+}
+
+// FP64 arithmetic: the digit products of gauss64.cu, then the sum over the splits
+static lsq_status gauss64_run(lsq_ctx* ctx, const lsq_matrix* A, int m, uint64_t seed, uint32_t t, double* SA,
+                              int64_t grow0) {
+  LsqGauss64 g;
+  const lsq_status st = lsq_gauss64_run(ctx, A, m, seed, t, grow0, &g);
+  if (st != LSQ_OK) return st;
+  const int64_t md = (int64_t)m * A->d;
+  reduce_splits_kernel<double><<<grid_for(md, 256, 4 * ctx->sm_count), 256, 0, ctx->stream>>>(
+      g.part, g.splits, md, 1.0 / sqrt((double)m), SA);
   LSQ_LAUNCH_CHECK();
   return LSQ_OK;
 }
@@ -1651,8 +1649,8 @@ static lsq_status sketch_impl(lsq_ctx* ctx, const lsq_matrix* A, int32_t type, i
     case LSQ_SKETCH_GAUSS:
       if (prec == LSQ_SKETCH_BF16)
         st = lsq_gauss_tc_run(ctx, A, (int)m, seed, t, SA, up ? chunk_upload : nullptr, up ? &cu : nullptr, row0);
-      else st = f64 ? gauss_run<double>(ctx, A, (int)m, seed, t, SA, row0)
-                    : gauss_run<float>(ctx, A, (int)m, seed, t, SA, row0);
+      else st = f64 ? gauss64_run(ctx, A, (int)m, seed, t, SA, row0)
+                    : gauss_run(ctx, A, (int)m, seed, t, SA, row0);
       break;
     case LSQ_SKETCH_SRHT:
       st = f64 ? srht_run<double>(ctx, A, (int)m, seed, t, SA, a32, ld32, a32_done, up, row0, n_total)

@@ -1,0 +1,69 @@
+"""The FP64 Gaussian sketch from digit products against the FP64 oracle: every entry of S (A = I), sizes
+around its tiles (64 x 64), stages (16 rows) and folds (128 rows), FP32 and strided A, columns over
++-1e100 with outlier rows, a row slab, and non-finite entries.
+
+Bound: an entry of S differs from the oracle's by the errors of two FP64 evaluations (log, square root,
+sine: a few units of 2^-53 each, the angle 2 pi u2 rounded once more) and 2^-58: below 1e-14 absolute; a
+column of SA by sqrt(n) 2^-57 of its norm on top, below 1e-14 relative for the sizes here."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from gpu_util import to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    import paper_1911_02675_gb300 as lib
+    return lib
+
+
+@pytest.fixture(scope="module")
+def ctx(L):
+    c = L.Context(0)
+    yield c
+    c.close()
+
+
+def test_entries(L, ctx):
+    n, m = 700, 130
+    S = L.lsq_sketch(ctx, torch.eye(n, dtype=torch.float64, device="cuda"), "gauss", m, 11, t=3).cpu().numpy()
+    ref = O.sketch_gauss(np.eye(n), m, 11, 3)
+    assert np.abs(S - ref).max() * np.sqrt(m) < 1e-14
+
+
+@pytest.mark.parametrize("n,d,m,dtype,pad", [(1, 1, 1, np.float64, 0), (15, 3, 2, np.float64, 1),
+                                             (129, 64, 63, np.float64, 0), (1000, 65, 64, np.float32, 3),
+                                             (2049, 33, 65, np.float64, 0), (5000, 130, 200, np.float64, 2)])
+def test_sketch(L, ctx, n, d, m, dtype, pad):
+    g = np.random.default_rng(n)
+    A = g.standard_normal((n, d))
+    A[g.random(n) < 0.05] *= 100.0
+    A = (A * 10.0 ** g.uniform(-18, 18, size=d)).astype(dtype) if dtype == np.float32 else A * 10.0 ** g.uniform(-100, 100, size=d)
+    wide = to_dev(np.concatenate([A, np.full((n, pad), np.nan, dtype=dtype)], axis=1))
+    SA = L.lsq_sketch(ctx, wide[:, :d], "gauss", m, 5, t=1).cpu().numpy()
+    ref = O.sketch_gauss(A.astype(np.float64), m, 5, 1)
+    s = np.abs(ref).max(0)
+    assert (np.linalg.norm((SA - ref) / s, axis=0) / np.linalg.norm(ref / s, axis=0)).max() < 1e-14
+    if n >= 1000:
+        k = 512
+        top = L.lsq_sketch(ctx, wide[:k, :d], "gauss", m, 5, t=1, row0=0, n_total=n).cpu().numpy()
+        bot = L.lsq_sketch(ctx, wide[k:, :d], "gauss", m, 5, t=1, row0=k, n_total=n).cpu().numpy()
+        assert (np.linalg.norm((top + bot - ref) / s, axis=0) / np.linalg.norm(ref / s, axis=0)).max() < 1e-14
+
+
+def test_non_finite(L, ctx):
+    A = np.random.default_rng(3).standard_normal((300, 5))
+    clean = L.lsq_sketch(ctx, to_dev(A), "gauss", 70, 2).cpu().numpy()
+    E = np.zeros((300, 1))
+    E[40] = 1.0
+    z = O.sketch_gauss(E, 70, 2, 0)[:, 0]
+    A[40, 1], A[7, 2], A[40, 3], A[41, 3] = np.inf, np.nan, np.inf, -np.inf
+    SA = L.lsq_sketch(ctx, to_dev(A), "gauss", 70, 2).cpu().numpy()
+    assert np.array_equal(SA[:, [0, 4]], clean[:, [0, 4]])
+    assert np.array_equal(SA[:, 1], np.sign(z) * np.inf)
+    assert np.isnan(SA[:, 2]).all()
+    assert not np.isfinite(SA[:, 3]).any()
