@@ -25,7 +25,7 @@ namespace {
 
 constexpr int GT = 256;                 // threads of the product kernel: 8 warps of 16 x 16 outputs
 constexpr int BA = 64, BB = 32;         // its tile of H_S
-constexpr int KC = 16;                  // rows of SA per stage
+constexpr int KC = 32;                  // rows of SA per stage (of 16: 3% slower at 4096 x 1024)
 constexpr int FOLD = 128;               // rows between folds
 constexpr int PA = BA + 8, PB = BB + 8;  // row pitches in shared memory (16-byte pieces of 8 rows: distinct banks)
 
@@ -97,21 +97,24 @@ __global__ void __launch_bounds__(GT, 1) gram_mma_kernel(const uint16_t* __restr
     __syncthreads();
     if (k + KC < k1) load(k + KC, st ^ 1);
     asm volatile("cp.async.commit_group;" ::: "memory");
-    const uint16_t* As = sm + st * ST + lr * PA + wa + lc;
-    const uint16_t* Bs = sm + st * ST + SA_E + br * PB + wb + bc;
-    uint32_t b[NS][4];
 #pragma unroll
-    for (int j = 0; j < NS; ++j) ldsm4t(b[j], Bs + j * KC * PB);
+    for (int ks = 0; ks < KC; ks += 16) {
+      const uint16_t* As = sm + st * ST + (ks + lr) * PA + wa + lc;
+      const uint16_t* Bs = sm + st * ST + SA_E + (ks + br) * PB + wb + bc;
+      uint32_t b[NS][4];
 #pragma unroll
-    for (int i = 0; i < NS; ++i) {
-      uint32_t a[4];
-      ldsm4t(a, As + i * KC * PA);
+      for (int j = 0; j < NS; ++j) ldsm4t(b[j], Bs + j * KC * PB);
 #pragma unroll
-      for (int j = 0; j < NS; ++j)
-        if (i + j < NS) {
-          mma_bf16_16816(acc[i + j][0], a, b[j][0], b[j][1]);
-          mma_bf16_16816(acc[i + j][1], a, b[j][2], b[j][3]);
-        }
+      for (int i = 0; i < NS; ++i) {
+        uint32_t a[4];
+        ldsm4t(a, As + i * KC * PA);
+#pragma unroll
+        for (int j = 0; j < NS; ++j)
+          if (i + j < NS) {
+            mma_bf16_16816(acc[i + j][0], a, b[j][0], b[j][1]);
+            mma_bf16_16816(acc[i + j][1], a, b[j][2], b[j][3]);
+          }
+      }
     }
     since += KC;
     if (since == FOLD) {
