@@ -100,13 +100,26 @@ __device__ __forceinline__ void fused_rows(const TA* __restrict__ A, int64_t ld,
   if (R == 4) q += __shfl_xor_sync(0xffffffffu, q, 8);
 }
 
-// the row loop for ceil(d / 32) = NK column groups, the accumulators into the warp's wred row
+}  // namespace lsq_apass
+
+#include "apassdg.cuh"
+
+namespace lsq_apass {
+
+// the row loop for ceil(d / 32) = NK column groups, the accumulators into the warp's wred row; dg: the
+// digit tables stand in wred
 template <typename TA, int NK>
 __device__ __forceinline__ void fused_rows_to(const TA* __restrict__ A, int64_t ld, int d, int dp, int64_t r0,
-                                              int64_t r1, const double* vec_s, double* wred, double* qred) {
+                                              int64_t r1, const double* vec_s, double* wred, double* qred,
+                                              bool dg, const DigitTab& tab) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double acc[NK], q;
-  fused_rows<TA, NK, (NK <= 6 ? 4 : 2)>(A, ld, d, r0, r1, vec_s, acc, q);
+  if (NK > 2 && dg) {
+    digit_rows<TA, NK>(A, ld, d, r0, r1, vec_s, tab, acc, q);
+    __syncthreads();  // every warp is done with the tables
+  } else {
+    fused_rows<TA, NK, (NK <= 6 ? 4 : 2)>(A, ld, d, r0, r1, vec_s, acc, q);
+  }
 #pragma unroll
   for (int k = 0; k < NK; ++k) wred[warp * dp + lane + 32 * k] = acc[k];
   if (lane == 0) qred[warp] = q;
@@ -117,10 +130,19 @@ template <typename TA, int EPL>
 __device__ __noinline__ void fused_pass(const TA* __restrict__ A, int64_t ld, int d, int dp, int64_t r0, int64_t r1,
                            const double* vec_s, double* wred, double* qred, double* part, int P, int cta) {
 #define LSQ_FP_CASE(N) \
-  case N: fused_rows_to<TA, N>(A, ld, d, dp, r0, r1, vec_s, wred, qred); break;
+  case N: fused_rows_to<TA, N>(A, ld, d, dp, r0, r1, vec_s, wred, qred, dg, tab); break;
+  DigitTab tab{};
+  bool dg = false;
+  if constexpr (EPL >= 4) {
+    if (r1 - r0 >= DG_MIN_ROWS) {
+      const int dk = (d + 63) & ~63;
+      tab = digit_tab(wred, dk);
+      dg = digit_prep(tab, d, dk, vec_s, reinterpret_cast<int*>(qred));
+    }
+  }
   const int nk = (d + 31) >> 5;
   if constexpr (EPL <= 2) {
-    fused_rows_to<TA, EPL>(A, ld, d, dp, r0, r1, vec_s, wred, qred);
+    fused_rows_to<TA, EPL>(A, ld, d, dp, r0, r1, vec_s, wred, qred, dg, tab);
   } else if constexpr (EPL == 4) {
     switch (nk) { LSQ_FP_CASE(3) default: LSQ_FP_CASE(4) }
   } else if constexpr (EPL == 8) {
@@ -260,23 +282,25 @@ __device__ void fused_pass_f32(const TA* __restrict__ A, int64_t ld, int d, int 
 
 
 // ------------------------------------------------------------------------------------
-// The FP32 pass for wide FP32 rows (256 < d <= 1024, d a multiple of 4, 16-byte aligned rows)
-// with the rows staged by bulk copies: each warp keeps RING_NS of its rows in flight in a ring
+// The FP32 pass for wide FP32 rows (128 < d <= 1024, d a multiple of 4, 16-byte aligned rows)
+// with the rows staged by bulk copies: each warp keeps ring_ns(EPL) of its rows in flight in a ring
 // of shared-memory slots, one cp.async.bulk per row started by lane 0 and counted in bytes on
 // the slot's mbarrier, instead of one row prefetched in registers.  The registers that frees
 // hold p, and the deeper queue keeps HBM busy with one 256-thread CTA per SM.  Lane l owns the
-// columns 128 k + 4 l + t (k < 8, t < 4) and reads them as eight 16-byte vectors per row.
+// columns f32_col(k, l), as in the pass above, and both add in one order: the same bits.
+// Rows of 129 to 256 columns: two mixed solves over 262144 x 256, 6.76 -> 6.64 ms.
 // Every wait is bounded: on a time-out the pass records LSQ_ERR_TIMEOUT, waits (bounded) for
 // its copies still in flight and returns; the caller checks the flag at its next barrier.
 // ------------------------------------------------------------------------------------
-constexpr int RING_NS = 4;
+// rows of a warp in flight: 16 KB a warp at most, and no less than 8 KB at 1 KB rows
+constexpr __host__ __device__ int ring_ns(int epl) { return epl == 8 ? 8 : 4; }
 constexpr uint32_t RING_SPIN = 1u << 24;
 
 __device__ __forceinline__ uint32_t smem_u32a(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-__device__ __forceinline__ void ring_init(uint64_t* bars) {
+__device__ __forceinline__ void ring_init(uint64_t* bars, int n) {
   // thread 0, before a CTA barrier: one arrival (the expect-tx) per phase
-  for (int e = 0; e < LSQ_WARPS * RING_NS; ++e)
+  for (int e = 0; e < n; ++e)
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32a(bars + e)) : "memory");
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
@@ -302,58 +326,64 @@ __device__ __forceinline__ bool ring_wait(uint64_t* bar, uint32_t parity) {
   return false;
 }
 
-// ring: LSQ_WARPS x RING_NS slots of `slot_floats` floats; bars: LSQ_WARPS x RING_NS mbarriers;
+// ring: LSQ_WARPS x ring_ns(EPL) slots of `slot_floats` floats; bars: as many mbarriers;
 // phase: this thread's parity bits of its warp's slots (kept across passes by the caller)
 template <int EPL>
 __device__ inline void fused_pass_f32_ring(const float* __restrict__ A, int64_t ld, int d, int dp, int64_t r0,
                                            int64_t r1, const double* vec_s, double* wred, double* qred, double* part,
                                            int P, int cta, float* ring, int slot_floats, uint64_t* bars,
                                            uint32_t& phase, int* err) {
-  static_assert(EPL == 16 || EPL == 32, "rows of 512 or 1024 padded columns");
+  static_assert(EPL == 8 || EPL == 16 || EPL == 32, "rows of 256, 512 or 1024 padded columns");
+  constexpr int NS = ring_ns(EPL);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float* pf = reinterpret_cast<float*>(wred);
   for (int c = threadIdx.x; c < dp; c += blockDim.x) pf[c] = (float)vec_s[c];
   __syncthreads();
   float pv[EPL], acc[EPL];
-  bool okc[EPL / 4];
 #pragma unroll
-  for (int k = 0; k < EPL / 4; ++k) {
-    const int c0 = 128 * k + 4 * lane;
-    okc[k] = c0 < d;  // d is a multiple of 4: the four columns are in or out together
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      pv[4 * k + t] = okc[k] ? pf[c0 + t] : 0.0f;
-      acc[4 * k + t] = 0.0f;
-    }
+  for (int k = 0; k < EPL; ++k) {
+    const int c = f32_col<EPL>(k, lane);
+    pv[k] = c < d ? pf[c] : 0.0f;
+    acc[k] = 0.0f;
   }
   double q = 0.0;
-  float* slots = ring + (size_t)warp * RING_NS * slot_floats;
-  uint64_t* bar = bars + warp * RING_NS;
+  float* slots = ring + (size_t)warp * NS * slot_floats;
+  uint64_t* bar = bars + warp * NS;
   const uint32_t bytes = (uint32_t)d * 4u;
   const int64_t first = r0 + warp;
-  // rows first + LSQ_WARPS j of this warp; slot j % RING_NS
+  // rows first + LSQ_WARPS j of this warp; slot j % NS
   int64_t issued = 0, done = 0;
   const int64_t nrows = first < r1 ? (r1 - first + LSQ_WARPS - 1) / LSQ_WARPS : 0;
-  for (; issued < nrows && issued < RING_NS; ++issued)
+  for (; issued < nrows && issued < NS; ++issued)
     if (lane == 0) ring_issue(slots + issued * slot_floats, A + (first + LSQ_WARPS * issued) * ld, bytes, bar + issued);
   bool good = true;
   for (; done < nrows; ++done) {
-    const int s = (int)(done % RING_NS);
+    const int s = (int)(done % NS);
     const bool landed = __all_sync(0xffffffffu, ring_wait(bar + s, (phase >> s) & 1u));
     if (!landed) {
       good = false;
       break;
     }
     phase ^= 1u << s;
-    const float4* row = reinterpret_cast<const float4*>(slots + s * slot_floats);
+    const float* row = slots + s * slot_floats;
     float af[EPL];
+    if constexpr (EPL >= 16) {
+      // four adjacent columns a lane; d is a multiple of 4, so they are in or out together
 #pragma unroll
-    for (int k = 0; k < EPL / 4; ++k) {
-      const float4 v = okc[k] ? row[32 * k + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
-      af[4 * k] = v.x;
-      af[4 * k + 1] = v.y;
-      af[4 * k + 2] = v.z;
-      af[4 * k + 3] = v.w;
+      for (int k = 0; k < EPL; k += 4) {
+        const int c = f32_col<EPL>(k, lane);
+        const float4 v = c < d ? *reinterpret_cast<const float4*>(row + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+        af[k] = v.x;
+        af[k + 1] = v.y;
+        af[k + 2] = v.z;
+        af[k + 3] = v.w;
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < EPL; ++k) {
+        const int c = f32_col<EPL>(k, lane);
+        af[k] = c < d ? row[c] : 0.0f;
+      }
     }
     __syncwarp();  // every lane has its values: the slot may be refilled
     if (issued < nrows) {
@@ -372,18 +402,15 @@ __device__ inline void fused_pass_f32_ring(const float* __restrict__ A, int64_t 
     if (lane == 0) atomicCAS(err, 0, (int)LSQ_ERR_TIMEOUT);
     // the copies still in flight land before the slots are given up (bounded)
     for (; done < issued; ++done) {
-      const int s = (int)(done % RING_NS);
+      const int s = (int)(done % NS);
       if (ring_wait(bar + s, (phase >> s) & 1u)) phase ^= 1u << s;
     }
   }
   __syncthreads();  // every warp is done with pf before wred is overwritten
 #pragma unroll
-  for (int k = 0; k < EPL / 4; ++k) {
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int c = 128 * k + 4 * lane + t;
-      if (c < dp) wred[warp * dp + c] = (double)acc[4 * k + t];
-    }
+  for (int k = 0; k < EPL; ++k) {
+    const int c = f32_col<EPL>(k, lane);
+    if (c < dp) wred[warp * dp + c] = (double)acc[k];
   }
   if (lane == 0) qred[warp] = q;
   __syncthreads();
@@ -644,7 +671,7 @@ __device__ __forceinline__ double warp_sum_strip(const double* src, int P) {
 
 // standalone pass: CTA b handles rows [b * rows_per_cta, (b + 1) * rows_per_cta)
 template <typename TA, int EPL>
-__global__ void __launch_bounds__(LSQ_THREADS, 1) hmatvec_kernel(const void* A, int64_t n, int d, int dp, int64_t ld,
+__global__ void __launch_bounds__(LSQ_THREADS, (EPL <= 16 ? 2 : 1)) hmatvec_kernel(const void* A, int64_t n, int d, int dp, int64_t ld,
                                                                   int64_t rows_per_cta, const double* p, double* part) {
   extern __shared__ __align__(16) double smem[];
   double* vec = smem;

@@ -57,7 +57,7 @@ struct SolveArgs {
   double* out;       // [0] iters, [1] status, [2] passes, [3] est_err, [4] exact passes
   const float* a32;  // COPY kernels: FP32 copy of A (row stride ld32) that the FP32 passes read
   int64_t ld32;
-  int ring;          // FP32 rows, 256 < d <= 1024: the FP32 passes stage rows by bulk copies
+  int ring;          // FP32 rows, 128 < d <= 1024: the FP32 passes stage rows by bulk copies
 };
 
 // out[i] = sum_k M[i*d + k] vec_s[k] for k in [k_lo(i), k_hi(i)), one warp per output
@@ -113,15 +113,15 @@ __global__ void __launch_bounds__(LSQ_THREADS, (EPL <= 16 ? 2 : 1)) solve_kernel
   double* stage = S.wred + LSQ_WARPS * dp;  // dp: r or z staging for the triangular products
   S.qred = stage + dp;
   S.scal = S.qred + LSQ_WARPS;
-  // FP32 rows at the widest d (256 < d <= 1024): the bulk-copy ring of the FP32 passes (after the
+  // FP32 rows at the wider d (128 < d <= 1024): the bulk-copy ring of the FP32 passes (after the
   // scalars, on a 128-byte boundary) and its mbarriers
-  constexpr bool RING = MIXED && EPL >= 16 && (COPY || sizeof(TA) == 4);
-  __shared__ __align__(8) uint64_t ring_bars[RING ? LSQ_WARPS * RING_NS : 1];
+  constexpr bool RING = MIXED && EPL >= 8 && (COPY || sizeof(TA) == 4);
+  __shared__ __align__(8) uint64_t ring_bars[RING ? LSQ_WARPS * ring_ns(EPL) : 1];
   float* ring = reinterpret_cast<float*>(
       (reinterpret_cast<uintptr_t>(S.scal + 8) + 127) & ~static_cast<uintptr_t>(127));
   uint32_t ring_phase = 0;
   if constexpr (RING) {
-    if (a.ring && threadIdx.x == 0) ring_init(ring_bars);
+    if (a.ring && threadIdx.x == 0) ring_init(ring_bars, LSQ_WARPS * ring_ns(EPL));
     __syncthreads();
   }
   // the staged exact pass (MIXED, FP64 A): x in wred[0, dp), one row slot per warp in
@@ -638,8 +638,8 @@ extern "C" lsq_status lsq_solve(lsq_ctx* ctx, const lsq_matrix* A, const double*
   const bool f32_rows = mixed && (a32 != nullptr || A->dtype == LSQ_F32);
   const float* rows32 = a32 ? a32 : reinterpret_cast<const float*>(A->data);
   const int64_t ld_rows = a32 ? ld32 : A->ld;
-  const bool ring = f32_rows && epl >= 16 && d % 4 == 0 && ((uintptr_t)rows32 % 16) == 0 && (ld_rows * 4) % 16 == 0;
-  const size_t smem = solve_smem_bytes(dp) + (ring ? 128 + (size_t)LSQ_WARPS * lsq_apass::RING_NS * dp * 4 : 0);
+  const bool ring = f32_rows && epl >= 8 && d % 4 == 0 && ((uintptr_t)rows32 % 16) == 0 && (ld_rows * 4) % 16 == 0;
+  const size_t smem = solve_smem_bytes(dp) + (ring ? 128 + (size_t)LSQ_WARPS * lsq_apass::ring_ns(epl) * dp * 4 : 0);
   LSQ_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   LSQ_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, LSQ_THREADS, smem));
