@@ -114,12 +114,15 @@ __device__ __forceinline__ void fused_rows_to(const TA* __restrict__ A, int64_t 
                                               bool dg, const DigitTab& tab) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double acc[NK], q;
-  if (NK > 2 && dg) {
-    digit_rows<TA, NK>(A, ld, d, r0, r1, vec_s, tab, acc, q);
-    __syncthreads();  // every warp is done with the tables
-  } else {
-    fused_rows<TA, NK, (NK <= 6 ? 4 : 2)>(A, ld, d, r0, r1, vec_s, acc, q);
+  bool done = false;
+  if constexpr (digit_pass<TA, (NK + 1) / 2 * 2>()) {
+    if (dg) {
+      digit_rows<NK>(A, ld, d, r0, r1, vec_s, tab, acc, q);
+      __syncthreads();  // every warp is done with the tables
+      done = true;
+    }
   }
+  if (!done) fused_rows<TA, NK, (NK <= 6 ? 4 : 2)>(A, ld, d, r0, r1, vec_s, acc, q);
 #pragma unroll
   for (int k = 0; k < NK; ++k) wred[warp * dp + lane + 32 * k] = acc[k];
   if (lane == 0) qred[warp] = q;
@@ -133,9 +136,9 @@ __device__ __noinline__ void fused_pass(const TA* __restrict__ A, int64_t ld, in
   case N: fused_rows_to<TA, N>(A, ld, d, dp, r0, r1, vec_s, wred, qred, dg, tab); break;
   DigitTab tab{};
   bool dg = false;
-  if constexpr (EPL >= 4) {
+  if constexpr (digit_pass<TA, EPL>()) {
     if (r1 - r0 >= DG_MIN_ROWS) {
-      const int dk = (d + 63) & ~63;
+      const int dk = (d + 31) & ~31;
       tab = digit_tab(wred, dk);
       dg = digit_prep(tab, d, dk, vec_s, reinterpret_cast<int*>(qred));
     }

@@ -1,5 +1,5 @@
-"""The FP64 pass with its dot products from digit products (384 rows a CTA and more, d > 64), against
-extended precision: chunks of 64 columns and their remainders, tiles of 16 rows and theirs, both types,
+"""The FP64 pass with its dot products from digit products (FP64 rows of 65 to 512 columns, 192 and
+more a CTA; the other calls here keep FP64 sums), against extended precision: chunks of 32 columns and their remainders, tiles of 16 rows and theirs, both types,
 strided rows, rows and columns of very different scales, zeros, subnormals, entries of p out of the digits'
 range, infinities and NaNs.  Each v_j is a sum of n products a_ij w_i of d-term sums: with FP64
 accumulators of n / (152 x 8) rows at most and a few hundred partial sums, the error is below
