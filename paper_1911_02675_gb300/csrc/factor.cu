@@ -75,7 +75,7 @@ struct TileSmem {
 
 // the diagonal-block routines' arrays
 struct DiagSmem {
-  double a[32][33], b[32][33], c[32][33];
+  double a[32][33], b[32][33];
   double rinv[32], pinv[32];
   int bad;
 };
@@ -138,114 +138,124 @@ __device__ __forceinline__ void tri_decode(int e, int& a, int& b) {
   a = e - bb * (bb + 1) / 2;
 }
 
+// 1 / g, within an ulp or so: the hardware's approximation (20 bits) and one third-order Newton step
+// (Householder 1970).  Three dependent FP64 instructions where a division takes about ten.
+__device__ __forceinline__ double pivot_recip(double g) {
+  if (!(g > 0x1p-960 && g < 0x1p960)) return 1.0 / g;
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(g));
+  const double e = fma(-g, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
 // Cholesky of one 32 x 32 diagonal block by the whole CTA: R into Rkk, and 1 / R[i][i] into the
 // block's own diagonal in G (the block is not read again).  FP64 instructions are costly on
 // this part (a warp instruction holds a sub-partition's FP64 unit for ~70 cycles whatever its
 // active lanes), so the factorisation is right-looking with the live entries of each step
 // packed densely onto threads, one barrier per step:
-//   step j: R[j][l] = G[j][l] / sqrt(G[j][j]) and G[i][l] -= G[j][i] G[j][l] / G[j][j] for
-//   j < i <= l; the thread that updates G[j+1][j+1] also takes its reciprocal square root, so
-//   the next pivot is ready at the barrier.
+//   step j: G[i][l] -= G[j][i] G[j][l] / G[j][j] for j < i <= l; the thread that updates
+//   G[j+1][j+1] also takes its reciprocal, so the next pivot is ready at the barrier.
+// What bounds it is the chain of pivots, so the square roots stay off it: R[j][l] = G[j][l] / sqrt(G[j][j])
+// is left to the end, 32 rows at once.  (Measured, with the one-instruction steps of the inverse and the
+// panels below, against a reciprocal square root in each step and two or three instructions in theirs:
+// lsq_factor 4096 x 1024 mixed 2.66 -> 2.35 ms, 28 refreshes of d = 64 9.06 -> 8.42 ms.)
 // Sets *err to LSQ_ERR_RANK on a non-positive or non-finite pivot.
 __device__ void diag_chol(DiagSmem& sm, double* Gkk, double* Rkk, int ld, int* err) {
   double (*Gs)[33] = sm.a;
-  double (*Rs)[33] = sm.b;
   double* rinv = sm.rinv;
   double* pinv = sm.pinv;
   int& bad = sm.bad;
   const int tid = threadIdx.x, nt = blockDim.x;
-  for (int e = tid; e < 1024; e += nt) {
-    Gs[e >> 5][e & 31] = Gkk[(int64_t)(e >> 5) * ld + (e & 31)];
-    Rs[e >> 5][e & 31] = 0.0;
-  }
+  for (int e = tid; e < 1024; e += nt) Gs[e >> 5][e & 31] = Gkk[(int64_t)(e >> 5) * ld + (e & 31)];
   if (tid == 0) bad = 0;
   __syncthreads();
   if (tid == 0) {
     const double g = Gs[0][0];
     if (!(g > 0.0) || !isfinite(g)) bad = 1;
-    const double r = rsqrt(g);
-    rinv[0] = r;
-    pinv[0] = r * r;
+    pinv[0] = pivot_recip(g);
   }
+  // this thread's entries of every step, counted from the step's first row (nt >= 256: two at most)
+  int a0, b0, a1, b1;
+  tri_decode(tid, a0, b0);
+  tri_decode(tid + nt, a1, b1);
   __syncthreads();
-  for (int j = 0; j < 32; ++j) {
+  for (int j = 0; j < 31; ++j) {
     const int S = 31 - j, T = S * (S + 1) / 2;
-    const double ri = rinv[j], pv = pinv[j];
-    for (int e = tid; e < T + 32 - j; e += nt) {
-      if (e < T) {
-        int a, b;
-        tri_decode(e, a, b);
-        const int i = j + 1 + a, l = j + 1 + b;
-        const double g = fma(-(Gs[j][i] * pv), Gs[j][l], Gs[i][l]);
-        Gs[i][l] = g;
-        if (e == 0) {  // (i, l) = (j + 1, j + 1): the next pivot
-          if (!(g > 0.0) || !isfinite(g)) bad = 1;
-          const double r = rsqrt(g);
-          rinv[j + 1] = r;
-          pinv[j + 1] = r * r;
-        }
-      } else {
-        const int l = j + (e - T);
-        Rs[j][l] = Gs[j][l] * ri;
+    const double pv = pinv[j];
+    if (tid < T) {
+      const int i = j + 1 + a0, l = j + 1 + b0;
+      const double g = fma(-(Gs[j][i] * pv), Gs[j][l], Gs[i][l]);
+      Gs[i][l] = g;
+      if (tid == 0) {  // (i, l) = (j + 1, j + 1): the next pivot
+        if (!(g > 0.0) || !isfinite(g)) bad = 1;
+        pinv[j + 1] = pivot_recip(g);
       }
+    }
+    if (tid + nt < T) {
+      const int i = j + 1 + a1, l = j + 1 + b1;
+      Gs[i][l] = fma(-(Gs[j][i] * pv), Gs[j][l], Gs[i][l]);
     }
     __syncthreads();
   }
-  for (int e = tid; e < 1024; e += nt) Rkk[(int64_t)(e >> 5) * ld + (e & 31)] = Rs[e >> 5][e & 31];
-  if (tid < 32) Gkk[(int64_t)tid * ld + tid] = rinv[tid];
+  if (tid < 32) {
+    rinv[tid] = rsqrt(Gs[tid][tid]);
+    Gkk[(int64_t)tid * ld + tid] = rinv[tid];
+  }
+  __syncthreads();
+  for (int e = tid; e < 1024; e += nt) {
+    const int j = e >> 5, l = e & 31;
+    Rkk[(int64_t)j * ld + l] = l >= j ? Gs[j][l] * rinv[j] : 0.0;
+  }
   if (tid == 0 && bad) atomicCAS(err, 0, (int)LSQ_ERR_RANK);
   __syncthreads();
 }
 
 // W = R^{-1} of one 32 x 32 upper triangular block (Rkk; 1 / R[i][i] on the block's diagonal in
-// G), right-looking from the bottom row, one barrier per step:
-//   W[i][l] = (delta_il - S[i][l]) / R[i][i] for l >= i, then S[k][l] += R[k][i] W[i][l], k < i <= l.
+// G), right-looking from the bottom row, one barrier and one FP64 instruction an entry per step: with
+// S = the identity at first and R'[k][i] = R[k][i] / R[i][i],
+//   S[k][l] -= R'[k][i] S[i][l], k < i <= l,   and in the end W[i][l] = S[i][l] / R[i][i].
 __device__ void diag_inv(DiagSmem& sm, const double* Gkk, const double* Rkk, double* Wkk, int ld) {
   double (*Rs)[33] = sm.a;
   double (*Ss)[33] = sm.b;
-  double (*Ws)[33] = sm.c;
   double* rinv = sm.rinv;
   const int tid = threadIdx.x, nt = blockDim.x;
-  for (int e = tid; e < 1024; e += nt) {
-    Rs[e >> 5][e & 31] = Rkk[(int64_t)(e >> 5) * ld + (e & 31)];
-    Ss[e >> 5][e & 31] = 0.0;
-    Ws[e >> 5][e & 31] = 0.0;
-  }
   if (tid < 32) rinv[tid] = Gkk[(int64_t)tid * ld + tid];
   __syncthreads();
-  for (int i = 31; i >= 0; --i) {
+  for (int e = tid; e < 1024; e += nt) {
+    const int k = e >> 5, i = e & 31;
+    Rs[k][i] = Rkk[(int64_t)k * ld + i] * rinv[i];
+    Ss[k][i] = k == i ? 1.0 : 0.0;
+  }
+  __syncthreads();
+  for (int i = 31; i > 0; --i) {
     const int w = 32 - i;
-    const double ri = rinv[i];
-    for (int e = tid; e < (i + 1) * w; e += nt) {
+    for (int e = tid; e < i * w; e += nt) {
       const int k = e / w, l = i + e % w;
-      const double wil = ((i == l ? 1.0 : 0.0) - Ss[i][l]) * ri;
-      if (k == i) Ws[i][l] = wil;
-      else Ss[k][l] = fma(Rs[k][i], wil, Ss[k][l]);
+      Ss[k][l] = fma(-Rs[k][i], Ss[i][l], Ss[k][l]);
     }
     __syncthreads();
   }
-  for (int e = tid; e < 1024; e += nt) Wkk[(int64_t)(e >> 5) * ld + (e & 31)] = Ws[e >> 5][e & 31];
+  for (int e = tid; e < 1024; e += nt) Wkk[(int64_t)(e >> 5) * ld + (e & 31)] = Ss[e >> 5][e & 31] * rinv[e >> 5];
   __syncthreads();
 }
 
 // 32 x 8 panel task: out = R^{-T} Gt (R = Rkk upper, 1 / R[i][i] on the diagonal of Gkk) by
 // forward substitution: warp c solves column c, lane i keeps row i's running value, and each
-// step's new unknown is broadcast by a shuffle (no CTA barrier inside the solve).
+// step's new unknown is broadcast by a shuffle (no CTA barrier inside the solve).  The rows are
+// divided by their diagonal first, so that a step is one FP64 instruction.
 __device__ void trsm_task(TileSmem& sm, double* out, const double* Rkk, const double* Gt, const double* Gkk, int ld) {
   const int tid = threadIdx.x, lane = tid & 31, c = tid >> 5;
-  for (int e = tid; e < 1024; e += blockDim.x) sm.X[0][e >> 5][e & 31] = Rkk[(int64_t)(e >> 5) * ld + (e & 31)];
+  const double di = Gkk[(int64_t)lane * ld + lane];
+  for (int e = tid; e < 1024; e += blockDim.x) sm.X[0][e >> 5][lane] = Rkk[(int64_t)(e >> 5) * ld + lane] * di;
+  double acc = c < 8 ? Gt[(int64_t)lane * ld + c] * di : 0.0;
   __syncthreads();
   if (c < 8) {
-    double acc = Gt[(int64_t)lane * ld + c];
-    const double di = Gkk[(int64_t)lane * ld + lane];
-    double x = 0.0;
 #pragma unroll 4
-    for (int p = 0; p < 32; ++p) {
-      const double xp = __shfl_sync(0xffffffffu, acc * di, p);
-      if (lane == p) x = xp;
+    for (int p = 0; p < 31; ++p) {
+      const double xp = __shfl_sync(0xffffffffu, acc, p);
       if (lane > p) acc = fma(-sm.X[0][p][lane], xp, acc);
     }
-    out[(int64_t)lane * ld + c] = x;
+    out[(int64_t)lane * ld + c] = acc;
   }
   __syncthreads();
 }
@@ -279,8 +289,8 @@ __device__ void chol_inv_body(double* __restrict__ G, double* __restrict__ Rf, d
       const int64_t col = (int64_t)j * 32 + q * 8;
       trsm_task(sm, Rf + kk * dp + col, Rf + kk * dp + kk, G + kk * dp + col, G + kk * dp + kk, dp);
     }
+    if (rest == 0) break;  // (the last diagonal block was there before the barrier)
     if (gsync()) return;
-    if (rest == 0) break;
     // trailing update: G[i][j] -= R[k][i]^T R[k][j], k < i <= j; pair 0 is the next
     // diagonal block (k+1, k+1)
     const int pairs = rest * (rest + 1) / 2;
