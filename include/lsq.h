@@ -204,7 +204,8 @@ LSQ_API lsq_status lsq_upload_sketch(lsq_ctx* ctx, const void* host_A, int64_t h
  * paragraph; Section 6, which allows either a QR of SA or a Cholesky factor of H_S).
  *   SA : device, m x d FP64 (row-major), m >= d.
  *   R  : device, d x d FP64 output: upper triangular, positive diagonal, R^T R = H_S
- *        (Gram from exact digit products, rounded once to FP64, then Cholesky); the strict lower triangle is written as 0.
+ *        (Gram from exact digit products, rounded once to FP64, then Cholesky); the
+ *        strict lower triangle is written as 0.
  *   W  : device, d x d FP64 output: W = R^{-1} (upper triangular), which lsq_solve
  *        uses to apply H_S^{-1} r = W (W^T r) as two parallel triangular products.
  * Status LSQ_ERR_RANK (after a synchronisation) if a pivot is not positive. This call
