@@ -216,7 +216,8 @@ __global__ void __launch_bounds__(T, 1) gauss64_kernel(const uint16_t* __restric
       const int j = j0 + wa + g + (x >> 1) * 8, col = c0 + wb + c * 8 + 2 * tq + (x & 1);
       if (j < m && col < d) {
         const int e = (int)(mag[col] >> 20);
-        double v = fma((double)hi[c][x], 4294967296.0, (double)lo[c][x]) * pow2(max(e, 1) - 1086);
+        // (two factors: e - 1086 alone lies below the smallest power for columns under 2^-1011)
+        double v = fma((double)hi[c][x], 4294967296.0, (double)lo[c][x]) * 0x1p-58 * pow2(max(e, 1) - 1028);
         if (e == 0x7FF) {
           v = 0.0;
           for (int k = k0; k < k1 && i0 + k < n; ++k) {

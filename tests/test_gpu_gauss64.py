@@ -55,6 +55,16 @@ def test_sketch(L, ctx, n, d, m, dtype, pad):
         assert (np.linalg.norm((top + bot - ref) / s, axis=0) / np.linalg.norm(ref / s, axis=0)).max() < 1e-14
 
 
+def test_columns_near_the_smallest_numbers(L, ctx):
+    # entries of SA down to the subnormals: the bound of the columns above plus half a unit of 2^-1074
+    # for the rounding of each entry here and in the oracle's sums (300 of them)
+    A = np.random.default_rng(4).standard_normal((300, 6)) * np.array([1e-306, 3e-310, 0.0, 1e-305, 2.0 ** -1010, 1.0])
+    SA = L.lsq_sketch(ctx, to_dev(A), "gauss", 70, 2).cpu().numpy()
+    ref = O.sketch_gauss(A, 70, 2, 0)
+    assert (np.abs(ref).max(0) > 0).tolist() == [True, True, False, True, True, True]
+    assert np.all(np.abs(SA - ref) <= 1e-14 * np.abs(ref).max(0) * 10 + 301 * 2.0 ** -1074)
+
+
 def test_non_finite(L, ctx):
     A = np.random.default_rng(3).standard_normal((300, 5))
     clean = L.lsq_sketch(ctx, to_dev(A), "gauss", 70, 2).cpu().numpy()
