@@ -51,10 +51,16 @@ __device__ void fill_tables(Tables& tb) {
   }
 }
 
+// the uniform (k + 1/2) 2^-53 of a word pair, evaluated in FP64, as a multiple of 2^-54: from k = 2^52 on,
+// k + 1/2 has 54 bits and rounds to the even neighbour (at the top to 1)
+__device__ __forceinline__ unsigned long long uniform54(uint32_t hi, uint32_t lo) {
+  const unsigned long long k = (((unsigned long long)hi << 32) | lo) >> 11;
+  return 2 * k + ((hi >> 31) ? 2 * (k & 1ull) : 1ull);
+}
+
 // z(2q, i) and z(2q + 1, i) from the words of Philox(i, q, t, TAG_GAUSS)
 __device__ __forceinline__ void normal_pair(const Tables& tb, uint4 w, double& zc, double& zs) {
-  const unsigned long long k1 = ((((unsigned long long)w.x << 32) | w.y) >> 11) * 2 + 1;  // u1 2^54
-  const unsigned long long k2 = ((((unsigned long long)w.z << 32) | w.w) >> 11) * 2 + 1;  // u2 2^54
+  const unsigned long long k1 = uniform54(w.x, w.y), k2 = uniform54(w.z, w.w);  // 53 bits at most each
   // -2 ln u1: u1 = m 2^e, m c = 1 + r
   const int lz = __clzll((long long)k1);
   const unsigned long long n1 = k1 << lz;
@@ -79,9 +85,9 @@ __device__ __forceinline__ void normal_pair(const Tables& tb, uint4 w, double& z
   h = fma(h, e, h);
   e = fma(-g, h, 0.5);
   g = fma(g, e, g);
-  const double rad = fma(fma(-g, g, x), h, g);
+  const double rad = lz > 9 ? fma(fma(-g, g, x), h, g) : 0.0;  // (lz = 9: u1 rounded to 1, x = 0)
   // sine and cosine of 2 pi u2 from the middle of its 64th of a turn
-  const double2 sc = tb.sc[(int)(k2 >> 48)];
+  const double2 sc = tb.sc[(int)(k2 >> 48) & 63];  // (u2 rounded to 1 is a whole turn)
   const double a = (__longlong_as_double(0x4330000000000000ll | (long long)(k2 & 0xFFFFFFFFFFFFull)) - (0x1p52 + 0x1p47)) *
                    (6.28318530717958647692 * 0x1p-54);
   const double a2 = a * a;

@@ -65,6 +65,16 @@ def test_columns_near_the_smallest_numbers(L, ctx):
     assert np.all(np.abs(SA - ref) <= 1e-14 * np.abs(ref).max(0) * 10 + 301 * 2.0 ** -1074)
 
 
+def test_uniform_next_to_one(L, ctx):
+    # row 847055 of this instance draws u1 = 1 - 1.7e-10, where -2 ln u1 hangs on the last bit of u1;
+    # 32 rows of ones around it, each entry within 1e-14
+    i0, n = 847040, 1 << 20
+    SA = L.lsq_sketch(ctx, torch.ones((32, 1), dtype=torch.float64, device="cuda"), "gauss", 2, 11, t=3, row0=i0,
+                      n_total=n).cpu().numpy()[:, 0]
+    ref = [sum(O.gauss_z(11, 3, j, i) for i in range(i0, i0 + 32)) / np.sqrt(2) for j in (0, 1)]
+    assert np.abs(SA - ref).max() < 32e-14
+
+
 def test_non_finite(L, ctx):
     A = np.random.default_rng(3).standard_normal((300, 5))
     clean = L.lsq_sketch(ctx, to_dev(A), "gauss", 70, 2).cpu().numpy()
