@@ -15,9 +15,12 @@
 // that the 8 columns collect the sums over i + k = s of bytes i of A and digits k of p (i + k > 7 lies
 // below 2^-59).  A product is at most 255 x 128 and 7 of them in 32 columns stay below 2^24: the FP32
 // accumulators are exact.  (The first byte is a digit + 128: 128 times the sum of p's digits comes off.)
-// Elements 2^-64 or more below the scale, zeros and subnormals among them, become 0; rows that hold an
+// Elements 2^-64 or more below the scale, zeros and subnormals among them, become 0, and so do those that
+// meet a zero of p (they would set the scale of products that do not exist; 600011 x 333 with 64 zeros in
+// p, 619 us, with 111 of them everywhere 667); rows that hold an
 // infinity or a NaN, or whose largest product is outside 2^-796 ... 2^854, take FP64 arithmetic, and so
-// does the pass if p is not finite or its largest entry is outside 2^-600 ... 2^600.
+// does the pass if p is not finite, its largest entry is outside 2^-600 ... 2^600 or it has subnormal ones
+// (whose digits do not fill their scale).
 //
 // Bound by the FP64 pipe, now with one multiply-add an element and two instructions per 32 columns of 16
 // rows: 80% busy.  (The rest is the integer work of the digits, about 25 instructions an element, and
@@ -53,6 +56,7 @@ struct DigitTab {
   __half* dig;     // DG_ROWS x pitch: digits of p, in the order of epk
   int pitch;       // halves: 32 or 96 bytes past a multiple of 128, distinct banks for a half-warp's rows
   int lo;          // rows with E <= lo are left to FP64
+  uint32_t zeros;  // bit per 32 columns: some meet a zero of p, or lie past d
 };
 
 __device__ __forceinline__ DigitTab digit_tab(double* wred, int dk) {
@@ -62,10 +66,11 @@ __device__ __forceinline__ DigitTab digit_tab(double* wred, int dk) {
   t.dig = reinterpret_cast<__half*>(t.corr + dk / 4);
   t.pitch = dk + 16;
   t.lo = 0;
+  t.zeros = 0;
   return t;
 }
 
-// fills the tables from p (all threads); false if p is out of range.  red: 8 ints of scratch.
+// fills the tables from p (all threads); false if p is out of range.  red: 16 ints of scratch.
 __device__ inline bool digit_prep(DigitTab& t, int d, int dk, const double* vec_s, int* red) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t mx = 0;
@@ -77,6 +82,8 @@ __device__ inline bool digit_prep(DigitTab& t, int d, int dk, const double* vec_
     for (int r = 0; r < DG; ++r) t.dig[r * t.pitch + c] = __ushort_as_half(0);
     t.dig[(DG_ROWS - 1) * t.pitch + c] = __ushort_as_half(0);
   }
+  uint32_t zeros = 0;
+  bool sub = false;
   for (int ch = warp; ch < dk / 32; ch += LSQ_WARPS) {
     int sum[DG];
     {
@@ -84,12 +91,14 @@ __device__ inline bool digit_prep(DigitTab& t, int d, int dk, const double* vec_
       const double p = c < d ? vec_s[c] : 0.0;
       const uint32_t hi = (uint32_t)__double2hiint(p);
       const uint32_t ep = (hi >> 20) & 0x7FFu;
+      if (__any_sync(0xffffffffu, p == 0.0)) zeros |= 1u << ch;
+      sub |= ep == 0 && p != 0.0;
       long long T = (long long)((((unsigned long long)((hi & 0xFFFFFu) | (ep ? 0x100000u : 0u)) << 32) |
                                  (uint32_t)__double2loint(p)) << 1);
       if (hi >> 31) T = -T;
       const unsigned long long b = (unsigned long long)T + 0x0080808080808080ull;
       const int pos = (c & ~15) + 4 * (c & 3) + ((c >> 2) & 3);
-      t.epk[pos] = max(ep, p != 0.0 ? 1u : 0u) << 20;
+      t.epk[pos] = ep << 20;
 #pragma unroll
       for (int k = 0; k < DG; ++k) {
         const int D = (int)((uint32_t)(b >> (8 * (DG - 1 - k))) & 0xFFu) - 128;
@@ -106,14 +115,18 @@ __device__ inline bool digit_prep(DigitTab& t, int d, int dk, const double* vec_
       t.corr[8 * ch + lane] = 128 * v;
     }
   }
-  __syncthreads();
+  if (lane == 0) red[LSQ_WARPS + warp] = (int)zeros;
+  sub = __syncthreads_or(sub) != 0;
   uint32_t m = 0;
 #pragma unroll
-  for (int w = 0; w < LSQ_WARPS; ++w) m = max(m, (uint32_t)red[w]);
+  for (int w = 0; w < LSQ_WARPS; ++w) {
+    m = max(m, (uint32_t)red[w]);
+    t.zeros |= (uint32_t)red[LSQ_WARPS + w];
+  }
   __syncthreads();  // red is read before a warp leaves its q there
   const int e = (int)(m >> 20);
   t.lo = max(e + 64, 1250);
-  return e >= 1023 - 600 && e <= 1023 + 600;
+  return e >= 1023 - 600 && e <= 1023 + 600 && !sub;
 }
 
 constexpr int DG_HI = 2900;  // rows with E >= DG_HI are left to FP64
@@ -157,8 +170,7 @@ __device__ __forceinline__ void digit_load(double (&x)[8], double (&y)[8], const
 
 // the contribution of 32 columns to w: of row g in the even lanes, of row g + 8 in the odd ones; false
 // if a row's scale is out of range
-__device__ __forceinline__ bool digit_chunk(const double (&x)[8], const double (&y)[8], int c0, const DigitTab& t,
-                                            double& w) {
+__device__ __forceinline__ bool digit_chunk(double (&x)[8], double (&y)[8], int c0, const DigitTab& t, double& w) {
   const int lane = threadIdx.x & 31, g = lane >> 2, tq = lane & 3;
   uint32_t ep[8];
   {
@@ -166,6 +178,15 @@ __device__ __forceinline__ bool digit_chunk(const double (&x)[8], const double (
     const uint4 q1 = *reinterpret_cast<const uint4*>(t.epk + c0 + 16 + 4 * tq);
     ep[0] = q0.x; ep[1] = q0.y; ep[2] = q0.z; ep[3] = q0.w;
     ep[4] = q1.x; ep[5] = q1.y; ep[6] = q1.z; ep[7] = q1.w;
+  }
+  if ((t.zeros >> (c0 >> 5)) & 1u) {
+    // finite elements against a zero of p take no part; infinities and NaNs stay and are seen below
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (ep[i] == 0u) {
+        if (((uint32_t)__double2hiint(x[i]) & 0x7FFFFFFFu) < 0x7FF00000u) x[i] = 0.0;
+        if (((uint32_t)__double2hiint(y[i]) & 0x7FFFFFFFu) < 0x7FF00000u) y[i] = 0.0;
+      }
   }
   uint32_t k0 = 0, k1 = 0, m0 = 0, m1 = 0;
 #pragma unroll

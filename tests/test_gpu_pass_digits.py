@@ -84,6 +84,32 @@ def test_scales(kind):
     _check(A, p)
 
 
+@pytest.mark.parametrize("kind", ["zeros of p", "zeros past d", "subnormal p", "chunks of zeros"])
+def test_elements_that_meet_no_product(kind):
+    """The scale of a row and 32 columns comes from its products: neither from elements that meet a zero of
+    p (or lie past d), nor from subnormal entries of p; bounds as above."""
+    rng = np.random.default_rng(8)
+    d = 81
+    A, p = rng.standard_normal((N, d)), rng.standard_normal(d)
+    if kind == "zeros of p":
+        p *= 1e-125
+        p[[0, 40, 70]] = 0.0
+        A[:, [0, 40, 70]] *= 1e290
+    elif kind == "zeros past d":
+        p *= 1e-125
+        p[80] = 0.0
+        A[:, 80] *= 1e290
+    elif kind == "subnormal p":
+        p *= 1e-150
+        p[33] = 1e-320
+        A[:, :33] = A[:, 34:] = 0.0
+        A[:, 33] *= 1e200
+    else:
+        p[:64] = 0.0
+        A[::3, 64:] = 0.0
+    _check(A, p)
+
+
 @pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
 @pytest.mark.parametrize("where", ["A", "p"])
 def test_not_finite(bad, where):
