@@ -6,15 +6,17 @@
 // pass as p_j = T_j 2^(e_j - 1076), T_j an integer below 2^54 in 7 balanced base-256 digits.  The
 // elements of a row's 32 columns are put on one scale with the exponents of p taken in,
 // E = max (e(a_ij) + e_j):
-//   a_ij = U_ij 2^(E - e_j - 1084), |U_ij| < 2^62, 8 bytes,   a_ij p_j = U_ij T_j 2^(E - 2160),
+//   a_ij = U_ij 2^(E - e_j - 1084), |U_ij| < 2^62, 8 bytes and a sign,   a_ij p_j = U_ij T_j 2^(E - 2160),
 // so an element loses only what lies 2^-61 below the row's largest |a_ij p_j| there, whatever the
 // scales of rows and columns: w is at least as near to A p as with FP64 additions, which round at
 // 2^-53 of the partial sums.  The bytes of a 16 x 16 tile of A are formed in registers, in the layout
-// that an m16n8k16 MMA wants of its first operand, as FP16 subnormals (byte b is b 2^-24: byte
-// permutations, no arithmetic); the second operand of byte i holds in column s the digit s - i of p, so
-// that the 8 columns collect the sums over i + k = s of bytes i of A and digits k of p (i + k > 7 lies
-// below 2^-59).  A product is at most 255 x 128 and 7 of them in 32 columns stay below 2^24: the FP32
-// accumulators are exact.  (The first byte is a digit + 128: 128 times the sum of p's digits comes off.)
+// that an m16n8k16 MMA wants of its first operand, as FP16 subnormals (byte b is b 2^-24, with the sign of
+// its element: byte permutations, no arithmetic); the second operand of byte i holds in column s the digit
+// s - i of p, so that the 8 columns collect the sums over i + k = s of bytes i of A and digits k of p
+// (i + k > 7 lies below 2^-59).  A product is at most 255 x 128 and 7 of them in 32 columns stay below
+// 2^24: the FP32 accumulators are exact.  With signs and magnitudes (and not complements), elements that
+// fit their scale are exact whatever their sign, so sums of products that FP64 forms without rounding
+// (integers, A p = 0) are the same here: their nonzero bytes and digits have i + k <= 7.
 // Elements 2^-64 or more below the scale, zeros and subnormals among them, become 0, and so do those that
 // meet a zero of p (they would set the scale of products that do not exist; 600011 x 333 with 64 zeros in
 // p, 619 us, with 111 of them everywhere 667); rows that hold an
@@ -26,7 +28,7 @@
 // rows: 80% busy.  (The rest is the integer work of the digits, about 25 instructions an element, and
 // loads of 8 rows each, whose 8 cache lines take as many cycles: chunks of 64 columns, looked at twice,
 // spent more there than they saved in FP64.  More warps or rows prefetched into L2 gave nothing.)
-// Measured: 600011 x 333, FP64 sums 859 us, chunks of 64 columns 661, this 610; 1200011 x 160, 540 us.
+// Measured: 600011 x 333, FP64 sums 859 us, chunks of 64 columns 661, this 605; 1200011 x 160, 540 us.
 // FP32 rows keep FP64 sums (widening twice costs more: 1231 against 1618 us at 622592 x 301), and so do
 // rows of more than 512 columns (8 warps an SM, too few for both pipes: 1173 against 1323 us at
 // 311296 x 1000).
@@ -48,11 +50,10 @@ constexpr __host__ __device__ bool digit_pass() {
   return sizeof(TA) == 8 && EPL >= 4 && EPL <= 16;
 }
 
-// the tables, in the shared memory of the (not yet used) reduction buffer: 35 dk + 480 bytes of its
+// the tables, in the shared memory of the (not yet used) reduction buffer: 34 dk + 480 bytes of its
 // 64 dp, dk = d rounded up to 32
 struct DigitTab {
   uint32_t* epk;   // dk: exponent fields of p << 20, the columns of a lane's fragment adjacent
-  int* corr;       // dk / 32 x 8: what the first bytes' + 128 adds to the 8 sums of 32 columns
   __half* dig;     // DG_ROWS x pitch: digits of p, in the order of epk
   int pitch;       // halves: 32 or 96 bytes past a multiple of 128, distinct banks for a half-warp's rows
   int lo;          // rows with E <= lo are left to FP64
@@ -62,8 +63,7 @@ struct DigitTab {
 __device__ __forceinline__ DigitTab digit_tab(double* wred, int dk) {
   DigitTab t;
   t.epk = reinterpret_cast<uint32_t*>(wred);
-  t.corr = reinterpret_cast<int*>(t.epk + dk);
-  t.dig = reinterpret_cast<__half*>(t.corr + dk / 4);
+  t.dig = reinterpret_cast<__half*>(t.epk + dk);
   t.pitch = dk + 16;
   t.lo = 0;
   t.zeros = 0;
@@ -85,35 +85,21 @@ __device__ inline bool digit_prep(DigitTab& t, int d, int dk, const double* vec_
   uint32_t zeros = 0;
   bool sub = false;
   for (int ch = warp; ch < dk / 32; ch += LSQ_WARPS) {
-    int sum[DG];
-    {
-      const int c = 32 * ch + lane;
-      const double p = c < d ? vec_s[c] : 0.0;
-      const uint32_t hi = (uint32_t)__double2hiint(p);
-      const uint32_t ep = (hi >> 20) & 0x7FFu;
-      if (__any_sync(0xffffffffu, p == 0.0)) zeros |= 1u << ch;
-      sub |= ep == 0 && p != 0.0;
-      long long T = (long long)((((unsigned long long)((hi & 0xFFFFFu) | (ep ? 0x100000u : 0u)) << 32) |
-                                 (uint32_t)__double2loint(p)) << 1);
-      if (hi >> 31) T = -T;
-      const unsigned long long b = (unsigned long long)T + 0x0080808080808080ull;
-      const int pos = (c & ~15) + 4 * (c & 3) + ((c >> 2) & 3);
-      t.epk[pos] = ep << 20;
+    const int c = 32 * ch + lane;
+    const double p = c < d ? vec_s[c] : 0.0;
+    const uint32_t hi = (uint32_t)__double2hiint(p);
+    const uint32_t ep = (hi >> 20) & 0x7FFu;
+    if (__any_sync(0xffffffffu, p == 0.0)) zeros |= 1u << ch;
+    sub |= ep == 0 && p != 0.0;
+    long long T = (long long)((((unsigned long long)((hi & 0xFFFFFu) | (ep ? 0x100000u : 0u)) << 32) |
+                               (uint32_t)__double2loint(p)) << 1);
+    if (hi >> 31) T = -T;
+    const unsigned long long b = (unsigned long long)T + 0x0080808080808080ull;
+    const int pos = (c & ~15) + 4 * (c & 3) + ((c >> 2) & 3);
+    t.epk[pos] = ep << 20;
 #pragma unroll
-      for (int k = 0; k < DG; ++k) {
-        const int D = (int)((uint32_t)(b >> (8 * (DG - 1 - k))) & 0xFFu) - 128;
-        t.dig[(DG + k) * t.pitch + pos] = __int2half_rn(D);
-        sum[k] = D;
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < DG; ++k) sum[k] = __reduce_add_sync(0xffffffffu, sum[k]);
-    if (lane < 8) {
-      int v = 0;
-#pragma unroll
-      for (int k = 0; k < DG; ++k) v = k == lane ? sum[k] : v;
-      t.corr[8 * ch + lane] = 128 * v;
-    }
+    for (int k = 0; k < DG; ++k)
+      t.dig[(DG + k) * t.pitch + pos] = __int2half_rn((int)((uint32_t)(b >> (8 * (DG - 1 - k))) & 0xFFu) - 128);
   }
   if (lane == 0) red[LSQ_WARPS + warp] = (int)zeros;
   sub = __syncthreads_or(sub) != 0;
@@ -131,11 +117,9 @@ __device__ inline bool digit_prep(DigitTab& t, int d, int dk, const double* vec_
 
 constexpr int DG_HI = 2900;  // rows with E >= DG_HI are left to FP64
 
-// a, sh bits below the scale, as bytes: digit i in byte 7 - i, the first one + 128.  Negative elements
-// are complemented without the carry (2^-62 of the scale).
+// |a|, sh bits below the scale, as bytes: digit i in byte 7 - i
 __device__ __forceinline__ void digit_bytes(double a, int sh, uint32_t& u0, uint32_t& u1) {
   uint32_t hi = (uint32_t)__double2hiint(a), lo = (uint32_t)__double2loint(a);
-  const uint32_t neg = (uint32_t)((int)hi >> 31);
   hi = (hi & 0xFFFFFu) | 0x100000u;
   hi = __funnelshift_l(lo, hi, 9);
   lo <<= 9;
@@ -144,8 +128,13 @@ __device__ __forceinline__ void digit_bytes(double a, int sh, uint32_t& u0, uint
     hi = 0;
     sh -= 32;
   }
-  u0 = __funnelshift_rc(lo, hi, sh) ^ neg;
-  u1 = __funnelshift_rc(hi, 0u, sh) ^ neg ^ 0x80000000u;
+  u0 = __funnelshift_rc(lo, hi, sh);
+  u1 = __funnelshift_rc(hi, 0u, sh);
+}
+
+// the signs of two elements, in bits 15 and 31
+__device__ __forceinline__ uint32_t sign_pair(double a, double b) {
+  return __byte_perm((uint32_t)__double2hiint(a), (uint32_t)__double2hiint(b), 0x7030u) & 0x80008000u;
 }
 
 __device__ __forceinline__ void mma_f16_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
@@ -222,7 +211,9 @@ __device__ __forceinline__ bool digit_chunk(double (&x)[8], double (&y)[8], int 
       digit_bytes(x[i], (int)((F0 - ((uint32_t)__double2hiint(x[i]) & 0x7FFFFFFFu) - ep[i]) >> 20), x0[e], x1[e]);
       digit_bytes(y[i], (int)((F1 - ((uint32_t)__double2hiint(y[i]) & 0x7FFFFFFFu) - ep[i]) >> 20), y0[e], y1[e]);
     }
-    // two bytes of two elements at a time, then each pair of bytes widened
+    const uint32_t s0 = sign_pair(x[4 * kt], x[4 * kt + 1]), s1 = sign_pair(y[4 * kt], y[4 * kt + 1]);
+    const uint32_t s2 = sign_pair(x[4 * kt + 2], x[4 * kt + 3]), s3 = sign_pair(y[4 * kt + 2], y[4 * kt + 3]);
+    // two bytes of two elements at a time, then each byte of the two with their signs
     const __half* dp = t.dig + (g + DG) * t.pitch + c0 + 16 * kt + 4 * tq;
 #pragma unroll
     for (int h = 0; h < 4; ++h) {  // bytes 2h, 2h + 1
@@ -233,19 +224,19 @@ __device__ __forceinline__ bool digit_chunk(double (&x)[8], double (&y)[8], int 
       const uint32_t p3 = h < 2 ? __byte_perm(y0[2], y0[3], sel) : __byte_perm(y1[2], y1[3], sel);
       const int i0 = 7 - 2 * h;  // digit of the even byte
       const uint2 b = *reinterpret_cast<const uint2*>(dp - i0 * t.pitch);
-      const uint32_t a[4] = {p0 & 0x00FF00FFu, p1 & 0x00FF00FFu, p2 & 0x00FF00FFu, p3 & 0x00FF00FFu};
+      const uint32_t a[4] = {__byte_perm(p0, s0, 0x7250u), __byte_perm(p1, s1, 0x7250u),
+                             __byte_perm(p2, s2, 0x7250u), __byte_perm(p3, s3, 0x7250u)};
       mma_f16_16816(acc, a, b.x, b.y);
       const uint2 b1 = *reinterpret_cast<const uint2*>(dp - (i0 - 1) * t.pitch);
-      const uint32_t a1[4] = {__byte_perm(p0, 0u, 0x4341u), __byte_perm(p1, 0u, 0x4341u),
-                              __byte_perm(p2, 0u, 0x4341u), __byte_perm(p3, 0u, 0x4341u)};
+      const uint32_t a1[4] = {__byte_perm(p0, s0, 0x7351u), __byte_perm(p1, s1, 0x7351u),
+                              __byte_perm(p2, s2, 0x7351u), __byte_perm(p3, s3, 0x7351u)};
       mma_f16_16816(acc, a1, b1.x, b1.y);
     }
   }
   // sums s = 2 tq, 2 tq + 1 of both rows as one integer each, below 2^32; then the lanes of a pair join
   // theirs, 2^16 apart, the even one for row g, the odd one for row g + 8
-  const int2 cr = *reinterpret_cast<const int2*>(t.corr + c0 / 4 + 2 * tq);
-  const long long X0 = (long long)(__float2int_rn(acc[0] * 16777216.f) - cr.x) * 256 + (__float2int_rn(acc[1] * 16777216.f) - cr.y);
-  const long long X1 = (long long)(__float2int_rn(acc[2] * 16777216.f) - cr.x) * 256 + (__float2int_rn(acc[3] * 16777216.f) - cr.y);
+  const long long X0 = (long long)__float2int_rn(acc[0] * 16777216.f) * 256 + __float2int_rn(acc[1] * 16777216.f);
+  const long long X1 = (long long)__float2int_rn(acc[2] * 16777216.f) * 256 + __float2int_rn(acc[3] * 16777216.f);
   const bool odd = tq & 1;
   const long long got = __shfl_xor_sync(0xffffffffu, odd ? X0 : X1, 1);
   const long long Y = odd ? (got << 16) + X1 : (X0 << 16) + got;

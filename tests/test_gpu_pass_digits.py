@@ -110,6 +110,24 @@ def test_elements_that_meet_no_product(kind):
     _check(A, p)
 
 
+@pytest.mark.parametrize("d", [70, 160, 333])
+def test_integers_are_exact(d):
+    """Small integers with signs: every product and sum is exact in FP64, and in the digits."""
+    rng = np.random.default_rng(d)
+    A, p = rng.integers(-9, 10, (N, d)).astype(float), rng.integers(-300, 301, d).astype(float)
+    v, q = _run(A, p)
+    w = A @ p
+    assert np.array_equal(v, A.T @ w) and q == w @ w
+
+
+def test_null_vector():
+    """A p = 0 exactly over integers, which the solvers see as q = 0."""
+    A = np.random.default_rng(5).integers(-9, 10, (N, 96)).astype(float)
+    A[:, 48:] = -A[:, :48]
+    v, q = _run(A, np.full(96, 3.0))
+    assert q == 0.0 and not v.any()
+
+
 @pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
 @pytest.mark.parametrize("where", ["A", "p"])
 def test_not_finite(bad, where):
