@@ -6,6 +6,8 @@
 
 #include <stdint.h>
 
+#include <algorithm>
+
 namespace lsq_digits {
 
 constexpr unsigned long long BIAS = 0x8080808080808080ull;  // T + BIAS holds the digits + 128 as bytes
@@ -44,26 +46,55 @@ __global__ void __launch_bounds__(256) column_max_kernel(const TA* __restrict__ 
 }
 
 // digits of rows [r0, r0 + rows) of A (zeros from n on): plane i at out + i rows dq, row pitch dq; two
-// columns a thread
-template <typename TA, int NS>
+// columns a thread, 64 columns a block and every 8 gridDim.y-th row.  Of each column's elements there,
+// counts[c] (zeroed before) counts those whose exponent is at most `gap` below the column's largest, and
+// with NZ counts[d + c] those that are not zero.
+template <typename TA, int NS, bool NZ>
 __global__ void __launch_bounds__(256) digits_kernel(const TA* __restrict__ A, int64_t n, int d, int64_t ld, int dq,
-                                                     int64_t r0, int rows, const uint32_t* __restrict__ mag,
-                                                     uint32_t* __restrict__ out) {
-  const int half = dq / 2;
+                                                     int64_t r0, int rows, const uint32_t* __restrict__ mag, int gap,
+                                                     uint32_t* __restrict__ counts, uint32_t* __restrict__ out) {
+  __shared__ uint32_t cnt[NZ ? 2 : 1][64];
+  const int half = dq / 2, p = 2 * (threadIdx.x & 31), c = blockIdx.x * 64 + p;
   const int64_t plane = (int64_t)rows * half;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < plane; e += (int64_t)gridDim.x * blockDim.x) {
-    const int r = (int)(e / half), c = 2 * (int)(e - (int64_t)r * half);
+  int emax[2], least[2];
+  uint32_t large[2] = {0u, 0u}, nonzero[2] = {0u, 0u};
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    emax[q] = c + q < d ? max((int)(mag[c + q] >> 20), 1) : 1;
+    least[q] = max(emax[q] - gap, 1);
+  }
+  for (int e = threadIdx.x; e < (NZ ? 128 : 64); e += 256) cnt[e >> 6][e & 63] = 0u;
+  for (int r = blockIdx.y * 8 + (threadIdx.x >> 5); r < rows; r += 8 * gridDim.y) {
     unsigned long long U[2];
 #pragma unroll
-    for (int q = 0; q < 2; ++q)
-      U[q] = r0 + r < n && c + q < d
-                 ? biased_digits((double)__ldg(A + (r0 + r) * ld + c + q), max((int)(mag[c + q] >> 20), 1))
-                 : BIAS;
-#pragma unroll
-    for (int i = 0; i < NS; ++i) {
-      out[i * plane + e] = digit_pair(U[0], U[1], i);
+    for (int q = 0; q < 2; ++q) {
+      const double x = r0 + r < n && c + q < d ? (double)__ldg(A + (r0 + r) * ld + c + q) : 0.0;
+      U[q] = biased_digits(x, emax[q]);
+      large[q] += (int)(((uint32_t)__double2hiint(x) >> 20) & 0x7FFu) >= least[q] ? 1u : 0u;
+      if (NZ) nonzero[q] += ((uint32_t)__double2hiint(x) << 1 | (uint32_t)__double2loint(x)) != 0u ? 1u : 0u;
     }
+#pragma unroll
+    for (int i = 0; i < NS; ++i) out[i * plane + (int64_t)r * half + c / 2] = digit_pair(U[0], U[1], i);
   }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 2; ++q) {
+    if (large[q]) atomicAdd(&cnt[0][p + q], large[q]);
+    if (NZ && nonzero[q]) atomicAdd(&cnt[NZ ? 1 : 0][p + q], nonzero[q]);
+  }
+  __syncthreads();
+  const int col = blockIdx.x * 64 + threadIdx.x;
+  if (threadIdx.x < 64 && col < d && counts) {
+#pragma unroll
+    for (int k = 0; k < (NZ ? 2 : 1); ++k)
+      if (cnt[k][threadIdx.x]) atomicAdd(counts + k * d + col, cnt[k][threadIdx.x]);
+  }
+}
+
+// its grid: a row a warp, at most eight blocks an SM
+inline dim3 lsq_digits_grid(int dq, int rows, int sm_count) {
+  const int gx = dq / 64;
+  return dim3((unsigned)gx, (unsigned)std::max(1, std::min((rows + 7) / 8, (8 * sm_count + gx - 1) / gx)));
 }
 
 __device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const void* p) {

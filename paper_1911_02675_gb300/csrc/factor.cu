@@ -441,7 +441,7 @@ extern "C" lsq_status lsq_factor_ex(lsq_ctx* ctx, const double* SA, int64_t m, i
 
   const size_t mat = (size_t)dp * dp;
   size_t need = lsq_align256((size_t)splits * mat * 8) + 4 * lsq_align256(mat * 8) + lsq_align256(gp.tiles.size() * 8) +
-                lsq_align256((size_t)di * 4) + lsq_align256(gp.plane_bytes) +
+                lsq_align256(gp.mag_words * 4) + lsq_align256(gp.plane_bytes) +
                 lsq_align256(std::max<size_t>(1, nodes.size()) * 16) + lsq_align256(level_start.size() * 4) +
                 lsq_align256(64);
   lsq_status st = lsq_ensure_scratch(ctx, need);
@@ -453,7 +453,7 @@ extern "C" lsq_status lsq_factor_ex(lsq_ctx* ctx, const double* SA, int64_t m, i
   double* Wf = cv.take<double>(mat);
   double* Tb = cv.take<double>(mat);
   int2* d_tiles = cv.take<int2>(gp.tiles.size());
-  uint32_t* mag = cv.take<uint32_t>(di);
+  uint32_t* mag = cv.take<uint32_t>(gp.mag_words);
   uint32_t* planes = cv.take<uint32_t>(gp.plane_bytes / 4);
   int4* d_nodes = cv.take<int4>(std::max<size_t>(1, nodes.size()));
   int* d_levels = cv.take<int>(level_start.size());

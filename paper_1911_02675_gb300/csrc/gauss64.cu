@@ -281,9 +281,8 @@ lsq_status run(lsq_ctx* ctx, const lsq_matrix* A, int m, uint64_t seed, uint32_t
   LSQ_CUDA_TRY(cudaFuncSetAttribute(gauss64_kernel<TA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM));
   for (int64_t i0 = 0; i0 < n; i0 += panel) {
     const int rows = (int)std::min<int64_t>(panel, (n - i0 + KC - 1) / KC * KC);
-    const int64_t pairs = (int64_t)rows * (dq / 2);
-    const int grid = (int)std::min<int64_t>((pairs + 255) / 256, 8 * (int64_t)ctx->sm_count);
-    digits_kernel<TA, NS><<<grid, 256, 0, s>>>(data, n, d, A->ld, dq, i0, rows, mag, planes);
+    digits_kernel<TA, NS, false>
+        <<<lsq_digits_grid(dq, rows, ctx->sm_count), 256, 0, s>>>(data, n, d, A->ld, dq, i0, rows, mag, 0, nullptr, planes);
     LSQ_LAUNCH_CHECK();
     gauss64_kernel<TA><<<dim3((unsigned)gx, (unsigned)gy, (unsigned)splits), T, SMEM, s>>>(
         reinterpret_cast<const uint16_t*>(planes), rows, dq, data, n, d, A->ld, m, seed, t, i0, grow0, rows_per_split, mag,

@@ -6,16 +6,25 @@
 // (|D| <= 128, exact in BF16):  SA[r][a] = sum_i D_i[r][a] 256^(7-i) 2^(e_a - 1084),  63 bits below the
 // largest element at NS = 8.  A product of two digits is at most 2^14, so the FP32 accumulators hold
 // the sum over 128 rows of every pair with the same i + j exactly (8 pairs x 128 x 2^14 = 2^24); pairs
-// with i + j >= NS are dropped (2^-57 of the columns' norms at NS = 8, 2^-49 at 7).  The sums are
-// folded into 64-bit integers every 128 rows, and one FP64 rounding per element follows: the result is
-// nearer to H_S than FP64 multiply-adds (NS = 8, LSQ_PREC_F64) and than double-FP32 ones (NS = 7,
-// LSQ_PREC_MIXED), with the columns' scale taken out, whatever the rows.
+// with i + j >= NS are dropped.  The sums are folded into 64-bit integers every 128 rows, and one FP64
+// rounding per element follows.
+//
+// What is dropped is on the scale of the columns' largest elements, M_a M_b: about 2^-62 M_a M_b sqrt(m)
+// at NS = 8 and 2^-54 at 7 (rms over random digits).  FP64 multiply-adds round at 2^-54 of the partial
+// sums, which is more as long as the products themselves are not far below M_a M_b.  So a column takes
+// digits only if more than 5/8 of its elements lie within 2^5 of its largest: two such columns share at
+// least a quarter of their rows, their products there are 2^-10 M_a M_b or more, and over 64 rows and
+// more the FP64 sums' own error is no smaller (double-FP32, LSQ_PREC_MIXED: the 45 bits of its
+// elements).  A tile with any other column (a few dominant rows, mostly zeros) is summed with FP64 or
+// double-FP32 multiply-adds as the precision asks (direct_tile).  The sketch of a matrix of many rows has
+// columns near N(0, s): 80% of their elements lie within the 2^5 at 4 s.
 //
 // Bound by the MMAs, NS (NS + 1) / 2 for each 16 x 8 x 16 product, and the latency of a stage.  Measured
 // (maximum, digits and product; before: FP64 or double-FP32 multiply-adds in tiles of 64 x 64):
 // 4096 x 1024 mixed 1100 -> 568 us, 1204 x 301 FP64 169 -> 49 us, 256 x 64 FP64 75 -> 19 us.
 #include <algorithm>
 
+#include "apass.cuh"
 #include "common.cuh"
 #include "digits.cuh"
 
@@ -29,13 +38,98 @@ constexpr int KC = 32;                  // rows of SA per stage (of 16: 3% slowe
 constexpr int FOLD = 128;               // rows between folds
 constexpr int PA = BA + 8, PB = BB + 8;  // row pitches in shared memory (16-byte pieces of 8 rows: distinct banks)
 
+constexpr int GAP = 4;                   // exponents below its largest element's at which an element counts as large
+constexpr int TK = 16;                   // rows of SA per step of direct_tile
+
+// exponent field of column c's largest element, 1 for zeros and subnormals
+__device__ __forceinline__ int column_exp(const uint32_t* mag, int c) { return max((int)(mag[c] >> 20), 1); }
+
+// 2^k as the scale of column c: NaN where the column is not finite, 0 past the last column
+__device__ __forceinline__ double column_scale(const uint32_t* mag, int c, int d, int k) {
+  if (c >= d) return 0.0;
+  return column_exp(mag, c) == 0x7FF ? __longlong_as_double(0x7FF8000000000000ll) : pow2(k);
+}
+
+// what brings a column whose largest element lies outside 2^-20 .. 2^50 into the range of FP32 products
+__device__ __forceinline__ int df_shift(const uint32_t* mag, int c, int d) {
+  const int e = c < d ? column_exp(mag, c) : 1023;
+  return e > 1073 ? 1073 - e : e < 1003 ? 1023 - e : 0;
+}
+
+// out (+)= the sum over rows [r0, r1) of SA for the tile at (a0, b0), by multiply-adds: FP64, or DF:
+// double-FP32 (elements split into a 21-bit head and the FP32 rounding of the rest, exact products, sums
+// as (head, tail) pairs).  Thread (ty, tx) owns rows
+// ty + 16 i and columns tx + 16 j of the tile.
+template <bool DF>
+__device__ __noinline__ void direct_tile(const double* __restrict__ SA, int d, int dp, int r0, int r1, int a0, int b0,
+                                         const uint32_t* __restrict__ mag, void* smem, int accumulate,
+                                         double* __restrict__ out) {
+  using E = typename std::conditional<DF, float2, double>::type;
+  E (*Xa)[BA] = reinterpret_cast<E (*)[BA]>(smem);
+  E (*Xb)[BB] = reinterpret_cast<E (*)[BB]>(Xa + TK);
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  double acc[4][2] = {};
+  float ah[4][2] = {}, al[4][2] = {};
+  for (int k0 = r0; k0 < r1; k0 += TK) {
+    __syncthreads();  // the rows before are no longer read
+    for (int e = threadIdx.x; e < TK * (BA + BB); e += GT) {
+      const int k = e / (BA + BB), p = e - k * (BA + BB);
+      const int c = p < BA ? a0 + p : b0 + p - BA;
+      const double v = k0 + k < r1 && c < d ? SA[(int64_t)(k0 + k) * d + c] : 0.0;
+      E* o = p < BA ? &Xa[k][p] : &Xb[k][p - BA];
+      if constexpr (DF) {
+        // (by the exponent fields; what leaves the range, or is subnormal, is zero)
+        const uint32_t hi = (uint32_t)__double2hiint(v);
+        const int ec = (int)((hi >> 20) & 0x7FFu), es = ec + df_shift(mag, c, d);
+        const double u = __hiloint2double((int)((hi & 0x800FFFFFu) | ((uint32_t)es << 20)), __double2loint(v));
+        lsq_apass::split_df(ec > 0 && es > 0 ? u : 0.0, o->x, o->y);
+      } else {
+        *o = v;
+      }
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int k = 0; k < TK; ++k) {
+      E x[4], y[2];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[i] = Xa[k][ty + 16 * i];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) y[j] = Xb[k][tx + 16 * j];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          if constexpr (DF) lsq_apass::df_fma(x[i].x, x[i].y, y[j].x, y[j].y, ah[i][j], al[i][j]);
+          else acc[i][j] = fma(x[i], y[j], acc[i][j]);
+        }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int a = a0 + ty + 16 * i, b = b0 + tx + 16 * j;
+      if (a < dp && b < dp) {
+        double v = acc[i][j];
+        if constexpr (DF)
+          v = ((double)ah[i][j] + (double)al[i][j]) * column_scale(mag, a, d, -df_shift(mag, a, d)) *
+              column_scale(mag, b, d, -df_shift(mag, b, d));
+        double* o = out + (int64_t)a * dp + b;
+        *o = accumulate ? *o + v : v;
+      }
+    }
+}
+
 // part[split][a][b] (+)= the sum over the split's rows of the panel, for one tile of H_S that meets its
-// upper triangle; planes as digits_kernel writes them (rows a multiple of KC)
+// upper triangle; planes as digits_kernel writes them for the panel's `rows` (a multiple of KC, `live` of
+// them in SA, the first one row row0), with its counts `large`
 template <int NS>
 __global__ void __launch_bounds__(GT, 1) gram_mma_kernel(const uint16_t* __restrict__ planes, int rows, int dq, int dp,
                                                          int rows_per_split, const int2* __restrict__ tiles,
-                                                         const uint32_t* __restrict__ mag, int d, int accumulate,
-                                                         double* __restrict__ part) {
+                                                         const uint32_t* __restrict__ mag,
+                                                         const uint32_t* __restrict__ large,
+                                                         const double* __restrict__ SA, int row0, int live, int d,
+                                                         int accumulate, double* __restrict__ part) {
   extern __shared__ __align__(16) uint16_t sm[];  // two stages of [NS][KC][PA] and [NS][KC][PB]
   constexpr int SA_E = NS * KC * PA, SB_E = NS * KC * PB, ST = SA_E + SB_E;
   const int2 tl = tiles[blockIdx.x];
@@ -44,6 +138,7 @@ __global__ void __launch_bounds__(GT, 1) gram_mma_kernel(const uint16_t* __restr
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int wa = (warp & 3) * 16, wb = (warp >> 2) * 16;
   const int64_t plane = (int64_t)rows * dq;
+  double* out = part + (int64_t)blockIdx.y * dp * dp;
   auto load = [&](int k, int st) {
     uint16_t* dst = sm + st * ST;
     for (int e = tid; e < NS * KC * (BA + BB) / 8; e += GT) {
@@ -91,6 +186,20 @@ __global__ void __launch_bounds__(GT, 1) gram_mma_kernel(const uint16_t* __restr
   const int br = (lane & 7) + ((lane >> 3) & 1) * 8, bc = ((lane >> 4) & 1) * 8;    // B: (k, n) 00 10 01 11
   if (k0 < k1) load(k0, 0);  // (a short last panel leaves splits empty)
   asm volatile("cp.async.commit_group;" ::: "memory");
+  bool uneven = false;  // (columns of zeros are exact either way, those with infinities or NaNs end as NaN)
+  if (tid < BA + BB) {
+    const int c = tid < BA ? a0 + tid : b0 + tid - BA;
+    if (c < d) {
+      const uint32_t m = mag[c];
+      uneven = m != 0u && m < 0x7FF00000u && 8ull * large[c] <= 5ull * (unsigned)live;
+    }
+  }
+  if (__syncthreads_or(uneven)) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");  // (direct_tile starts with a barrier)
+    direct_tile<NS < 8>(SA, d, dp, row0 + min(k0, live), row0 + min(k1, live), a0, b0, mag, sm, accumulate,
+                        out);
+    return;
+  }
   int since = 0;
   for (int k = k0, st = 0; k < k1; k += KC, st ^= 1) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -125,13 +234,7 @@ __global__ void __launch_bounds__(GT, 1) gram_mma_kernel(const uint16_t* __restr
   fold();
   // H_S[a][b] = (hi 2^32 + lo) 2^56 2^(e_a - 1084) 2^(e_b - 1084), NaN where a column is not finite
   const int g = lane >> 2, t = lane & 3;
-  double* out = part + (int64_t)blockIdx.y * dp * dp;
-  auto scale = [&](int c) -> double {
-    if (c >= d) return 0.0;
-    const int e = (int)(mag[c] >> 20);
-    if (e == 0x7FF) return __longlong_as_double(0x7FF8000000000000ll);
-    return pow2(max(e, 1) - 1084 + 28);
-  };
+  auto scale = [&](int c) { return column_scale(mag, c, d, c < d ? column_exp(mag, c) - 1084 + 28 : 0); };
 #pragma unroll
   for (int n = 0; n < 2; ++n)
 #pragma unroll
@@ -149,17 +252,19 @@ template <int NS>
 lsq_status run(lsq_ctx* ctx, const double* SA, int m, int d, int dp, int dq, int panel, int splits, int rows_per_split,
                const int2* d_tiles, int ntiles, uint32_t* mag, uint32_t* planes, double* part) {
   cudaStream_t s = ctx->stream;
+  uint32_t* large = mag + d;  // of each panel
   constexpr size_t smem = (size_t)2 * (NS * KC * PA + NS * KC * PB) * 2;
   LSQ_CUDA_TRY(cudaFuncSetAttribute(gram_mma_kernel<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   for (int r0 = 0; r0 < m; r0 += panel) {
     const int rows = std::min(panel, (m - r0 + KC - 1) / KC * KC);
-    const int64_t pairs = (int64_t)rows * (dq / 2);
-    const int grid = (int)std::min<int64_t>((pairs + 255) / 256, 8 * (int64_t)ctx->sm_count);
-    digits_kernel<double, NS><<<grid, 256, 0, s>>>(SA, m, d, d, dq, r0, rows, mag, planes);
+    const dim3 grid = lsq_digits_grid(dq, rows, ctx->sm_count);
+    digits_kernel<double, NS, false><<<grid, 256, 0, s>>>(SA, m, d, d, dq, r0, rows, mag, GAP, large, planes);
     LSQ_LAUNCH_CHECK();
     gram_mma_kernel<NS><<<dim3((unsigned)ntiles, (unsigned)splits), GT, smem, s>>>(
-        reinterpret_cast<const uint16_t*>(planes), rows, dq, dp, rows_per_split, d_tiles, mag, d, r0 > 0 ? 1 : 0, part);
+        reinterpret_cast<const uint16_t*>(planes), rows, dq, dp, rows_per_split, d_tiles, mag, large, SA, r0,
+        std::min(rows, m - r0), d, r0 > 0 ? 1 : 0, part);
     LSQ_LAUNCH_CHECK();
+    large += d;
   }
   return LSQ_OK;
 }
@@ -185,12 +290,13 @@ LsqGramPlan lsq_gram_plan(const lsq_ctx* ctx, int m, int d, bool mixed) {
   p.rows_per_split = ((p.panel + splits - 1) / splits + KC - 1) / KC * KC;
   p.splits = (p.panel + p.rows_per_split - 1) / p.rows_per_split;
   p.plane_bytes = (size_t)p.ns * p.panel * p.dq * 2;
+  p.mag_words = (size_t)d * (1 + (m + p.panel - 1) / p.panel);
   return p;
 }
 
 lsq_status lsq_gram_run(lsq_ctx* ctx, const LsqGramPlan& p, const double* SA, int m, int d, const int2* d_tiles,
                         uint32_t* mag, uint32_t* planes, double* part) {
-  LSQ_CUDA_TRY(cudaMemsetAsync(mag, 0, (size_t)d * 4, ctx->stream));
+  LSQ_CUDA_TRY(cudaMemsetAsync(mag, 0, p.mag_words * 4, ctx->stream));
   const int cb = (d + 31) / 32;
   const int rb = std::max(1, std::min((m + 7) / 8, (4 * ctx->sm_count + cb - 1) / cb));
   column_max_kernel<double><<<dim3((unsigned)cb, (unsigned)rb), 256, 0, ctx->stream>>>(SA, m, d, d, mag);

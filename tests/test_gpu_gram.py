@@ -46,6 +46,28 @@ def test_r_of_scaled_columns(L, ctx, m, d, precision):
     assert np.abs(WR - np.eye(d)).max() < 1e-9
 
 
+@pytest.mark.parametrize("precision", ["f64", "mixed"])
+@pytest.mark.parametrize("kind", ["even", "2^10", "2^20", "2^30", "sparse", "scaled"])
+def test_entries_where_columns_peak_in_different_rows(L, ctx, kind, precision):
+    """H_S[0][b] = R[0][0] R[0][b] entry by entry, on the scale of sum_r |a_r b_r| and not of the columns'
+    norms: FP64 multiply-adds err by at most m 2^-53 of it, double-FP32 ones by 2^-44 (45 bits of each
+    element) and m 2^-46 (the FP32 sums of their tails), and R[0][0], R[0][b] by a few units more."""
+    g = np.random.default_rng(11)
+    m, d = 1024, 70
+    X = g.standard_normal((m, d))
+    if kind == "sparse":
+        X *= g.random((m, d)) < 0.05
+    elif kind != "even":
+        X[(7 * np.arange(d)) % m, np.arange(d)] = 2.0 ** {"2^10": 10, "2^20": 20, "2^30": 30, "scaled": 20}[kind]
+    s = 10.0 ** g.uniform(-100, 100, size=d) if kind == "scaled" else np.ones(d)
+    R, _ = L.lsq_factor(ctx, to_dev(X * s), precision=precision)
+    X = (X * s).astype(np.longdouble)
+    H, S = X[:, 0] @ X, np.abs(X[:, 0]) @ np.abs(X)
+    got = R.cpu().numpy()[0].astype(np.longdouble)
+    u = m * 2.0 ** -53 if precision == "f64" else 2.0 ** -44 + m * 2.0 ** -46
+    assert np.all(np.abs(got[0] * got - H) <= (u + 8 * 2.0 ** -53) * S)
+
+
 @pytest.mark.parametrize("bad", [np.nan, np.inf])
 def test_non_finite_is_a_rank_error(L, ctx, bad):
     A = np.random.default_rng(1).standard_normal((300, 40))
