@@ -84,7 +84,7 @@ __global__ void __launch_bounds__(256) digits_kernel(const TA* __restrict__ A, i
   }
   __syncthreads();
   const int col = blockIdx.x * 64 + threadIdx.x;
-  if (threadIdx.x < 64 && col < d && counts) {
+  if (threadIdx.x < 64 && col < d) {
 #pragma unroll
     for (int k = 0; k < (NZ ? 2 : 1); ++k)
       if (cnt[k][threadIdx.x]) atomicAdd(counts + k * d + col, cnt[k][threadIdx.x]);

@@ -6,9 +6,16 @@
 // 2 MB of A are nothing.  Here a CTA owns a 64 x 64 tile of SA and a range of rows.  Per 16 rows it draws
 // its entries of S (table-driven log, sine and cosine with Taylor polynomials, a Goldschmidt square
 // root: ~40 FP64 instructions a pair), writes them as 8 base-256 digits in fixed point (2^-58) to shared
-// memory, and multiplies them with the digits of A's columns (columns in fixed point on the scale of their
+// memory, and multiplies them with the digits of A's columns (columns in fixed point on the scale M of their
 // largest element, digits_kernel): 36 digit products, each summed exactly in FP32 over 128 rows, then in
-// 64-bit integers.  S stays in shared memory.  The result is nearer to S A than FP64 multiply-adds.
+// 64-bit integers.  S stays in shared memory.
+//
+// An entry of SA differs from its value by about 2^-58 M sqrt(nonzero elements of the column) (digit pairs that
+// are dropped, S in fixed point).  FP64 rounds every z a at 2^-53 |z a| and the partial sums of its row splits,
+// which is more once the elements of M/8 and above are a 16th of the column's nonzero ones, or as many as
+// the splits (2 an SM); and with 16 of them no entry hangs on one small z.  A tile with a column that has
+// fewer (a few dominant rows) is summed in FP64, from FP64 Box-Muller entries (direct_tile).
+//
 // Bound by the FP64 pipe (Box-Muller).  Measured (the sketch's kernels before its last
 // reduction): 4096 x 64, m = 256: 219 -> 77 us; m = 512: 381 -> 130 us.
 #include <math.h>
@@ -28,6 +35,8 @@ constexpr int BM = 64, BN = 64, KC = 16, FOLD = 128;
 constexpr int PITCH = 64 + 8;        // row pitch in shared memory
 constexpr int OPER = NS * KC * PITCH;  // one operand's digits of a stage
 constexpr size_t SMEM = (size_t)4 * OPER * 2 + 128 * 16 + 64 * 16;
+
+constexpr int GAP = 2;                // exponents below its largest's at which an element of A counts as large
 
 struct Tables {
   double2 lg[128];  // c ~ 1 / m of the interval, 2 ln c
@@ -102,13 +111,69 @@ __device__ __forceinline__ void normal_pair(const Tables& tb, uint4 w, double& z
   zc = rad * (sc.y + fma(sc.y, cm, -(sc.x * sa)));
 }
 
+// out[j][c] (+)= sum over rows [i_begin, i_end) of z(j, i) A[i][c] for the tile at (j0, c0), in FP64
+template <typename TA>
+__device__ __noinline__ void direct_tile(const TA* __restrict__ A, int64_t i_begin, int64_t i_end, int d, int64_t ld, int m,
+                                         uint64_t seed, uint32_t t, int64_t grow0, int j0, int c0, void* smem,
+                                         int accumulate, double* __restrict__ out) {
+  double (*Ss)[BM] = reinterpret_cast<double (*)[BM]>(smem);
+  double (*As)[BN] = reinterpret_cast<double (*)[BN]>(Ss + KC);
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  double acc[4][4] = {};
+  for (int64_t i0 = i_begin; i0 < i_end; i0 += KC) {
+    __syncthreads();  // the rows before are no longer read
+    for (int e = threadIdx.x; e < KC * BM / 2; e += T) {
+      const int jp = e / KC, k = e % KC;
+      double zc = 0.0, zs = 0.0;
+      if (i0 + k < i_end) {
+        const uint4 w = philox_at(seed, (uint32_t)(i0 + k + grow0), (uint32_t)((j0 >> 1) + jp), t, TAG_GAUSS);
+        const double rad = sqrt(-2.0 * log((double)uniform54(w.x, w.y) * 0x1p-54));
+        double sn, cs;
+        sincospi((double)uniform54(w.z, w.w) * 0x1p-53, &sn, &cs);
+        zc = rad * cs;
+        zs = rad * sn;
+      }
+      Ss[k][2 * jp] = zc;
+      Ss[k][2 * jp + 1] = zs;
+    }
+    for (int e = threadIdx.x; e < KC * BN; e += T) {
+      const int k = e / BN, c = e % BN;
+      As[k][c] = i0 + k < i_end && c0 + c < d ? (double)__ldg(A + (i0 + k) * ld + c0 + c) : 0.0;
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int k = 0; k < KC; ++k) {
+      double s[4], a[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) s[r] = Ss[k][ty + 16 * r];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) a[c] = As[k][tx + 16 * c];
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[r][c] = fma(s[r], a[c], acc[r][c]);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int j = j0 + ty + 16 * r, col = c0 + tx + 16 * c;
+      if (j < m && col < d) {
+        double* o = out + (int64_t)j * d + col;
+        *o = accumulate ? *o + acc[r][c] : acc[r][c];
+      }
+    }
+}
+
 // part[split][j][c] (+)= sum over the split's rows of the panel of z(j, i) A[i][c]; planes: the digits of
-// the panel's rows (from row i0 of A, `rows` a multiple of KC)
+// the panel's rows (from row i0 of A, `rows` a multiple of KC), with their counts (digits_kernel)
 template <typename TA>
 __global__ void __launch_bounds__(T, 1) gauss64_kernel(const uint16_t* __restrict__ planes, int rows, int dq,
                                                        const TA* __restrict__ A, int64_t n, int d, int64_t ld, int m,
                                                        uint64_t seed, uint32_t t, int64_t i0, int64_t grow0,
                                                        int rows_per_split, const uint32_t* __restrict__ mag,
+                                                       const uint32_t* __restrict__ counts, uint32_t enough,
                                                        int accumulate, double* __restrict__ part) {
   extern __shared__ __align__(16) uint16_t sm[];  // [2] digits of S, [2] digits of A, tables
   Tables& tb = *reinterpret_cast<Tables*>(sm + 4 * OPER);
@@ -117,6 +182,7 @@ __global__ void __launch_bounds__(T, 1) gauss64_kernel(const uint16_t* __restric
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int wa = (warp & 3) * 16, wb = (warp >> 2) * 32;
   const int64_t plane = (int64_t)rows * dq;
+  double* out = part + (int64_t)blockIdx.z * m * d;
   auto load = [&](int k, int st) {
     uint16_t* dst = sm + (2 + st) * OPER;
     for (int e = tid; e < NS * KC * BN / 8; e += T) {
@@ -177,7 +243,17 @@ __global__ void __launch_bounds__(T, 1) gauss64_kernel(const uint16_t* __restric
   fill_tables(tb);
   if (k0 < k1) load(k0, 0);
   asm volatile("cp.async.commit_group;" ::: "memory");
-  __syncthreads();  // the tables are there
+  // (columns of zeros are exact either way; those with infinities or NaNs are seen at the end)
+  bool few = false;
+  if (tid < BN && c0 + tid < d) {
+    const uint32_t mg = mag[c0 + tid];
+    few = mg != 0u && mg < 0x7FF00000u && counts[c0 + tid] < max(16u, min(counts[d + c0 + tid] / 16u, enough));
+  }
+  if (__syncthreads_or(few)) {  // (the tables are there, too)
+    asm volatile("cp.async.wait_group 0;" ::: "memory");  // (direct_tile starts with a barrier)
+    direct_tile(A, i0 + k0, min(n, i0 + k1), d, ld, m, seed, t, grow0, j0, c0, sm, accumulate, out);
+    return;
+  }
   if (k0 < k1) draw(k0, 0);
   int since = 0;
   for (int k = k0, st = 0; k < k1; k += KC, st ^= 1) {
@@ -214,7 +290,6 @@ __global__ void __launch_bounds__(T, 1) gauss64_kernel(const uint16_t* __restric
   // (hi 2^32 + lo) 2^56 2^-58 2^(emax - 1084); a column with infinities or NaNs: what its non-finite
   // elements give in floating point
   const int g = lane >> 2, tq = lane & 3;
-  double* out = part + (int64_t)blockIdx.z * m * d;
 #pragma unroll
   for (int c = 0; c < 4; ++c)
 #pragma unroll
@@ -264,29 +339,32 @@ lsq_status run(lsq_ctx* ctx, const lsq_matrix* A, int m, uint64_t seed, uint32_t
   }
   const int rows_per_split = (int)((stages + splits - 1) / splits) * KC;
   splits = (panel + rows_per_split - 1) / rows_per_split;
+  // the columns' largest magnitudes, then the two counts of every panel
+  const int64_t mag_words = d * (1 + 2 * ((n + panel - 1) / panel));
   const size_t need = lsq_align256((size_t)splits * m * d * 8) + lsq_align256((size_t)NS * panel * dq * 2) +
-                      lsq_align256((size_t)d * 4);
+                      lsq_align256((size_t)mag_words * 4);
   lsq_status st = lsq_ensure_scratch(ctx, need);
   if (st != LSQ_OK) return st;
   Carver cv{reinterpret_cast<char*>(ctx->scratch), 0};
   double* part = cv.take<double>((size_t)splits * m * d);
   uint32_t* planes = cv.take<uint32_t>((size_t)NS * panel * dq / 2);
-  uint32_t* mag = cv.take<uint32_t>(d);
+  uint32_t* mag = cv.take<uint32_t>(mag_words);
   cudaStream_t s = ctx->stream;
-  LSQ_CUDA_TRY(cudaMemsetAsync(mag, 0, (size_t)d * 4, s));
+  LSQ_CUDA_TRY(cudaMemsetAsync(mag, 0, (size_t)mag_words * 4, s));
   const int cb = (d + 31) / 32;
   const int rb = (int)std::max<int64_t>(1, std::min<int64_t>((n + 7) / 8, (4 * ctx->sm_count + cb - 1) / cb));
   column_max_kernel<TA><<<dim3((unsigned)cb, (unsigned)rb), 256, 0, s>>>(data, n, d, A->ld, mag);
   LSQ_LAUNCH_CHECK();
   LSQ_CUDA_TRY(cudaFuncSetAttribute(gauss64_kernel<TA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM));
-  for (int64_t i0 = 0; i0 < n; i0 += panel) {
+  uint32_t* counts = mag + d;
+  for (int64_t i0 = 0; i0 < n; i0 += panel, counts += 2 * d) {
     const int rows = (int)std::min<int64_t>(panel, (n - i0 + KC - 1) / KC * KC);
-    digits_kernel<TA, NS, false>
-        <<<lsq_digits_grid(dq, rows, ctx->sm_count), 256, 0, s>>>(data, n, d, A->ld, dq, i0, rows, mag, 0, nullptr, planes);
+    digits_kernel<TA, NS, true>
+        <<<lsq_digits_grid(dq, rows, ctx->sm_count), 256, 0, s>>>(data, n, d, A->ld, dq, i0, rows, mag, GAP, counts, planes);
     LSQ_LAUNCH_CHECK();
     gauss64_kernel<TA><<<dim3((unsigned)gx, (unsigned)gy, (unsigned)splits), T, SMEM, s>>>(
         reinterpret_cast<const uint16_t*>(planes), rows, dq, data, n, d, A->ld, m, seed, t, i0, grow0, rows_per_split, mag,
-        i0 > 0 ? 1 : 0, part);
+        counts, 2u * ctx->sm_count, i0 > 0 ? 1 : 0, part);
     LSQ_LAUNCH_CHECK();
   }
   out->part = part;

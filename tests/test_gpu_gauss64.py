@@ -75,6 +75,42 @@ def test_uniform_next_to_one(L, ctx):
     assert np.abs(SA - ref).max() < 32e-14
 
 
+def _entries(m, n, seed, t):
+    """sqrt(m) S in extended precision, from the same uniforms"""
+    w = O.philox4x32_10([(i, j, t, 1) for i in range(n) for j in range(m // 2)], (seed, 0)).astype(np.uint64)
+    k1, k2 = ((w[:, 0] << 32 | w[:, 1]) >> 11), ((w[:, 2] << 32 | w[:, 3]) >> 11)
+    u1, u2 = ((k.astype(np.float64) + 0.5) * 2.0 ** -53 for k in (k1, k2))
+    pi = 4 * np.arctan(np.longdouble(1))
+    rad = np.sqrt(-2 * np.log(u1.astype(np.longdouble)))
+    h = np.rint(4 * u2)                                  # quarter turns, exact remainder
+    a = 2 * pi * (u2 - h / 4).astype(np.longdouble)
+    sn, cs = np.sin(a), np.cos(a)
+    h = h.astype(int) % 4
+    z = np.empty((m, n), dtype=np.longdouble)
+    z[0::2] = (rad * np.choose(h, [cs, -sn, -cs, sn])).reshape(n, m // 2).T
+    z[1::2] = (rad * np.choose(h, [sn, cs, -sn, -cs])).reshape(n, m // 2).T
+    return z
+
+
+@pytest.mark.parametrize("n,d", [(64, 3), (700, 67)])
+def test_entries_that_hang_on_one_row(L, ctx, n, d):
+    """Columns with one nonzero row, with one dominant row and even ones, entry by entry on the scale of
+    sum_i |z(j, i) a_i|: FP64 entries of S are within 8 units (logarithm, square root, sine, their
+    product), their products and sums within n."""
+    m = 400
+    g = np.random.default_rng(n)
+    A = g.standard_normal((n, d))
+    A[:, 0] = 0.0
+    A[:, d // 2] *= 1e-9
+    A[n // 3, [0, d // 2]] = 3.0
+    SA = L.lsq_sketch(ctx, to_dev(A), "gauss", m, 9, t=2).cpu().numpy()
+    z, A = _entries(m, n, 9, 2), A.astype(np.longdouble)
+    ref, S = z @ A, np.abs(z) @ np.abs(A)
+    err = np.abs(SA * np.sqrt(np.longdouble(m)) - ref)
+    assert np.all(err <= (2 * 8 + n + 4) * 2.0 ** -53 * S)
+    assert np.all(err[:, 0] <= (2 * 8 + 4) * 2.0 ** -53 * S[:, 0])
+
+
 def test_non_finite(L, ctx):
     A = np.random.default_rng(3).standard_normal((300, 5))
     clean = L.lsq_sketch(ctx, to_dev(A), "gauss", 70, 2).cpu().numpy()
