@@ -8,7 +8,8 @@
 //             all k_p directions at once; chunks of rows are taken from a queue (costliest
 //             first) by 512-thread CTAs; a tile of rows is staged in shared memory,
 //             Y = A_tile P (rows x k) and then V += A_tile^T Y, FP32 under LSQ_PREC_MIXED (over FP32 A
-//             on the tensor cores, bmma.cuh; exact residuals over FP32 A in btile.cuh), FP64 otherwise;
+//             with contiguous, 16-byte aligned rows on the tensor cores, bmma.cuh, with exact residuals in
+//             btile.cuh), FP64 otherwise;
 //   update    alpha_j = r_j^T z_j / q_j, x_j += alpha_j p_j, r_j -= alpha_j v_j (a warp per 32
 //             columns);
 //   precond   t = W^T r, then z = W t (W = R^{-1}), a CTA per 32 rows of W whose warps split the
@@ -239,11 +240,27 @@ __device__ __forceinline__ void pass_chunk(const BProb& pr, int64_t r0, int64_t 
         const int c0 = s_slice * cs;
         const TT* arow = As + r * dp;
         const int sw = (r & 7) << 2;
-        for (int c = c0; c < c0 + cs; ++c) {
-          const TT a = arow[c ^ sw];
-          const TT* pc = Ps + c * KP;
+        if constexpr (sizeof(TT) == 4 && TE == 16384) {
+          // cs = TE / BT = 32 columns: 8 groups of 4, each one 16-byte load of the row
 #pragma unroll
-          for (int j = 0; j < KP; ++j) y[j] = fma(a, pc[j], y[j]);
+          for (int g = 0; g < 8; ++g) {
+            const int c = c0 + 4 * g;
+            const float4 a4 = *reinterpret_cast<const float4*>(arow + (c ^ sw));
+            const float av[4] = {a4.x, a4.y, a4.z, a4.w};
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const TT* pc = Ps + (c + q) * KP;
+#pragma unroll
+              for (int j = 0; j < KP; ++j) y[j] = fma(av[q], pc[j], y[j]);
+            }
+          }
+        } else {
+          for (int c = c0; c < c0 + cs; ++c) {
+            const TT a = arow[c ^ sw];
+            const TT* pc = Ps + c * KP;
+#pragma unroll
+            for (int j = 0; j < KP; ++j) y[j] = fma(a, pc[j], y[j]);
+          }
         }
         if (S == 1) {
 #pragma unroll
@@ -493,7 +510,7 @@ constexpr int PT = 512;  // threads of a pass CTA (the other kernels use BT)
 
 // shared memory of the passes for one problem shape (the launch takes the maximum); mirrors
 // the layouts of pass_chunk and pass_chunk_df with PT threads
-__host__ __device__ inline size_t pass_smem_shape(bool mixed, int dp, int KP) {
+__host__ __device__ inline size_t pass_smem_shape(bool mixed, bool a_f64, int dp, int KP) {
   auto tile = [&](size_t es, int TE) {
     const int tr = TE / dp;
     const int S = tr >= PT ? 1 : PT / tr;
@@ -501,10 +518,10 @@ __host__ __device__ inline size_t pass_smem_shape(bool mixed, int dp, int KP) {
   };
   size_t f = 0;
   if (mixed) {
-    f = tile(4, 8192);
+    f = tile(4, a_f64 ? 8192 : 16384);
     const int TEd = 8192, trd = TEd / dp, Sd = trd >= PT ? 1 : PT / trd;
     const size_t df =
-        (size_t)(TEd * 2 + 2 * dp * KP + (Sd > 1 ? 2 * Sd * KP * trd : 0) + 2 * trd * KP) * 4;
+        (size_t)(TEd * (a_f64 ? 2 : 1) + 2 * dp * KP + (Sd > 1 ? 2 * Sd * KP * trd : 0) + 2 * trd * KP) * 4;
     f = f > df ? f : df;
   } else {
     f = tile(8, 8192);
@@ -520,11 +537,12 @@ __host__ __device__ inline size_t pass_smem_shape(bool mixed, int dp, int KP) {
 template <typename TA, bool MIXED>
 __device__ void pass_one(const BatchArgs& a, int ch, bool force_exact, int it, uint8_t* smem) {
   using TT = typename std::conditional<MIXED, float, double>::type;
-  constexpr int TEP = 8192;  // elements of a tile
+  // elements of a tile: 64 KB of FP32; 8192 when the tile or the prefetch is FP64
+  constexpr int TEP = (MIXED && sizeof(TA) == 4) ? 16384 : 8192;
   const int4 cd = a.chunks[ch];
   const BProb& pr = a.probs[cd.x];
   if (!prob_active(pr, it)) return;
-  if (pass_smem_shape(MIXED, pr.dp, pr.kp) > (size_t)a.smem_bytes) {
+  if (pass_smem_shape(MIXED, sizeof(TA) == 8, pr.dp, pr.kp) > (size_t)a.smem_bytes) {
     // the launch's shared memory does not hold this shape (cannot happen with the host's sizing)
     if (threadIdx.x == 0) atomicCAS(a.err, 0, (int)LSQ_ERR_ARG);
     return;
@@ -1121,11 +1139,15 @@ extern "C" lsq_status lsq_solve_batched(lsq_ctx* ctx, int32_t nprob, lsq_problem
   const ChunkPlan* plan = &plans[0];
 
   // ---- the pass kernel: dynamic shared memory for the largest problem shape
-  // FP32 A in the mixed precision: the tile pass of btile.cuh; otherwise the tiled pass above
-  const bool tile = dtype == LSQ_F32 && mixed;
+  // FP32 A in the mixed precision with contiguous, 16-byte aligned rows: the passes of btile.cuh and
+  // bmma.cuh; otherwise the tiled pass above (over FP32 A with FP32 multiply-adds, whose q_j is nearer to
+  // ||A p_j||^2 than the tensor cores' sums: 1e-8 against 3e-7 over 20000 rows of 33 to 512 columns)
+  bool tile = dtype == LSQ_F32 && mixed;
+  for (int p = 0; p < nprob && tile; ++p)
+    tile = probs[p].A.ld == probs[p].A.d && ((uintptr_t)probs[p].A.data % 16) == 0;
   void* kpass = tile ? (void*)btile_kernel
-                     : dtype == LSQ_F32 ? (void*)bpass_kernel<float, false>
-                                        : (mixed ? (void*)bpass_kernel<double, true> : (void*)bpass_kernel<double, false>);
+                     : dtype == LSQ_F64 ? (mixed ? (void*)bpass_kernel<double, true> : (void*)bpass_kernel<double, false>)
+                                        : (mixed ? (void*)bpass_kernel<float, true> : (void*)bpass_kernel<float, false>);
   const int pass_threads = tile ? TT : PT;
   size_t smem = 0;
   if (tile) {
@@ -1133,7 +1155,7 @@ extern "C" lsq_status lsq_solve_batched(lsq_ctx* ctx, int32_t nprob, lsq_problem
   } else {
     for (int p = 0; p < nprob; ++p) {
       const int dpp = dp_of((int)probs[p].A.d), kpp = kp_of(probs[p].k);
-      smem = std::max(smem, pass_smem_shape(mixed, dpp, kpp));
+      smem = std::max(smem, pass_smem_shape(mixed, dtype == LSQ_F64, dpp, kpp));
     }
   }
   if (smem > 227 * 1024) return LSQ_ERR_ARG;

@@ -19,8 +19,8 @@
 // row stride is 4 x odd: the columns of a k-step and the rows of a tile may be taken in any order,
 // so with a stride of 2 x odd (odd) the eight rows of a tile half lie 2 (4) apart, and the row pairs
 // of a k-step 4 (8).  That covers the rows as they lie in memory unless d is a multiple of 8; those
-// (and rows with a gap or off 16 bytes) are copied one by one to a stride 4 more than a multiple
-// of 8.
+// are copied one by one to a stride 4 more than a multiple of 8.  (Rows are contiguous and 16-byte
+// aligned: batch.cu sends other problems to the tiled pass.)
 //
 // Why warp-level MMAs: at HBM rate an SM has ~20 instructions per element and thread slot; FP32 FMAs
 // took 53 at 16 right-hand sides (packed two to an instruction) and ran at 1.2 TB/s, bound by issue
@@ -48,7 +48,7 @@ __device__ __forceinline__ MmaShape mma_shape(const BProb& pr) {
   s.lgks = s.kd <= 8 ? 0 : s.kd <= 16 ? 1 : s.kd <= 32 ? 2 : 3;
   s.R = 256 >> s.lgks;
   s.kps = (s.kd + (1 << s.lgks) - 1) >> s.lgks;
-  s.rows = d % 8 == 0 || pr.ld != d || ((uintptr_t)pr.A % 16) != 0;
+  s.rows = d % 8 == 0;
   s.stride = s.rows ? ((d + 3) & ~7) + 4 : d;
   s.lgm = s.rows || d % 4 == 0 ? 0 : d % 2 == 0 ? 1 : 2;
   return s;
@@ -106,33 +106,24 @@ __device__ __forceinline__ bool tm_chunk(const BProb& pr, int64_t r0, int64_t r1
   const int64_t ld = pr.ld;
   const int nst = (int)((r1 - r0 + R - 1) / R);
   bool ok = true;
-  // row-by-row copies: this thread's piece of a row (F floats from column lc) and its first row of a
-  // sweep of TT / pc rows
-  const int F = pr.vec ? 4 : (ld % 2 == 0 && ((uintptr_t)A % 8) == 0) ? 2 : 1;
-  const int pc = (d + F - 1) / F, lsweep = max(1, TT / pc), lrow = tid / pc, lc = (tid - lrow * pc) * F;
-  auto load_rows = [&](auto fc, int64_t lo, float* buf) {
-    constexpr int FC = decltype(fc)::value;
-    for (int c = lc; c < d; c += TT * FC) {  // (one trip unless a row has more than TT pieces)
-      const int nb = 4 * min(FC, d - c);
-      const float* src = A + (lo + lrow) * ld + c;
-      float* dst = buf + lrow * stride + c;
-      const int left = (int)min((int64_t)R, r1 - lo);
-      for (int r = lrow; r < R; r += lsweep) {
-        tp_copy<FC>(dst, r < left ? src : A, r < left ? nb : 0);
-        src += (int64_t)lsweep * ld;
-        dst += lsweep * stride;
-      }
+  // row-by-row copies: this thread's 4 columns of a row (from column lc) and its first row of a sweep of
+  // TT / pc rows (pc <= 128 pieces a row)
+  const int pc = max(1, d >> 2), lsweep = TT / pc, lrow = tid / pc, lc = (tid - lrow * pc) * 4;
+  auto load_rows = [&](int64_t lo, float* buf) {
+    const float* src = A + (lo + lrow) * ld + lc;
+    float* dst = buf + lrow * stride + lc;
+    const int left = (int)min((int64_t)R, r1 - lo);
+    for (int r = lrow; r < R; r += lsweep) {
+      tp_copy<4>(dst, r < left ? src : A, r < left ? 16 : 0);
+      src += (int64_t)lsweep * ld;
+      dst += lsweep * stride;
     }
   };
   auto load = [&](int t, int slot) {
     float* buf = stage0 + slot * sf;
     const int64_t lo = r0 + (int64_t)t * R;
     if (ms.rows) {
-      if (t < nst && lrow < lsweep) {
-        if (F == 4) load_rows(std::integral_constant<int, 4>{}, lo, buf);
-        else if (F == 2) load_rows(std::integral_constant<int, 2>{}, lo, buf);
-        else load_rows(std::integral_constant<int, 1>{}, lo, buf);
-      }
+      if (t < nst && lrow < lsweep) load_rows(lo, buf);
       asm volatile("cp.async.commit_group;" ::: "memory");
     } else if (t < nst && tid == 0) {
       // the stage's element range rounded out to 16 bytes; where that would read past the matrix the

@@ -62,3 +62,22 @@ def test_first_iterate(L, ctx, x0, layout):
         assert it == 1 and st == L.LSQ_ERR_MAXIT, (sh, it, st)
         start = X0[i] if x0 else 0.0
         assert rel_fro(Xp.cpu().numpy() - start, Xr - start) < 1e-5, sh
+
+
+@pytest.mark.parametrize("d,pad", [(33, 1), (64, 4), (255, 1), (512, 4)])
+def test_rows_with_gaps_keep_fp32_sums(L, ctx, d, pad):
+    """Batches whose rows have gaps take FP32 multiply-adds: the first iterate x = u <b, u> / ||A u||^2 shows
+    ||A p||^2, whose roundings (of p, and of 20000 sums of d products) are as often up as down and average
+    out below one unit of 2^-24 over the batch (the tensor cores' sums, cut off, lie 3e-7 low)."""
+    g = torch.Generator(device="cuda").manual_seed(d)
+    probs = []
+    for _ in range(16):
+        wide = torch.randn((20000, d + pad), generator=g, dtype=torch.float32, device="cuda")
+        probs.append((wide[:, :d], torch.randn((2, d), generator=g, dtype=torch.float64, device="cuda")))
+    X, _, _ = L.lsq_solve_batched(ctx, probs, tol=1e-12, maxit=1, precision="mixed", seed=4)
+    err = []
+    for (A, B), x in zip(probs, X):
+        for xj, b in zip(x, B):
+            u = xj / xj.norm()
+            err.append(float(xj.norm() * (A.double() @ u).square().sum() / (b @ u)) - 1.0)
+    assert np.sqrt(np.mean(np.square(err))) < 2.0 ** -24
