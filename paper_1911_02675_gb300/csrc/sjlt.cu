@@ -533,6 +533,24 @@ lsq_status lsq_sjlt_hash_launch(lsq_ctx* ctx, int64_t n, int m, int s, uint64_t 
   return LSQ_OK;
 }
 
+// Whether one matrix is gathered (else the scatter of sketch.cu).  The gather adds in registers, but sorts
+// n s entries and visits m targets a chunk, whatever d is: it wants many additions for its targets,
+// s n d >= 12 m^2, no more than 4096 sqrt(s) targets (every slice of 4096 reads A again, and a row's lists grow
+// with m / R) and more columns than a tile's 16, unless s is large or a wide chunk has few targets.  Embeddings
+// of 8 d rows at most are gathered at any n: up to 8192 rows the lists cost them 10 to 30 us, with half
+// the error.  Measured over 2400 sizes (n 2^11..2^20, d 4..1000, m 16..51200, s 1..32), scatter against
+// gather: 2^20 x 512 FP64, m = 2048, s = 8, 6.54 and 2.37 ms; 2^18 x 512, m = 16384, 2.45 and 2.56;
+// m = 51200, 3.40 and 9.03; 2^18 x 64, m = 51200, 0.87 and 1.75; 2^20 x 4, m = 16, 0.40 and 2.1;
+// 32768 x 4, m = 1024, 32 and 53 us; 8192 x 100, m = 8192, 42 and 112 us.
+bool lsq_sjlt_gathers(int64_t n, int d, int m, int s) {
+  if (d > 16 && s >= 4 && m <= 8 * d && m <= 4096) return true;
+  const double mm = (double)m * m, adds = (double)s * n * d;
+  if (mm > 16777216.0 * s) return false;
+  if (s > 16) return 4.0 * mm <= adds && m >= 4 * s;
+  if ((s < 4 ? 24.0 : 12.0) * mm > adds || adds < 4194304.0) return false;
+  return d > 16 || (d > 8 && n >= (1 << 19) && m >= 8 * s && m <= 1024);
+}
+
 // SA (m x d FP64) of one matrix; m <= 51200 (the list kernel's counts)
 lsq_status lsq_sjlt_f32(lsq_ctx* ctx, const lsq_matrix* A, int m, int s, uint64_t seed, uint32_t t, double* SA,
                         int64_t grow0) {

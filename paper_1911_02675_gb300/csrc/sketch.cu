@@ -3,7 +3,7 @@
 // Every kernel streams A once (Gaussian: once per 64-row slab of S) and generates its
 // randomness on the fly from Philox4x32-10; S is never stored.  Partial sums go to a
 // per-split scratch slab and a fixed-order reduction writes SA, so results repeat run
-// to run (FP64 SJLT: up to the order of its shared-memory additions; the FP32 one is in sjlt.cu).
+// to run (SJLT: up to the order of its shared-memory additions; the gathered FP32 one is in sjlt.cu).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <math.h>
@@ -15,12 +15,13 @@
 #include "common.cuh"
 #include "fix96.cuh"
 
-// sjlt.cu: the hash pass (target rows in draw order and the sign word of every row of A) and the
-// FP32 sketch
+// sjlt.cu: the hash pass (target rows in draw order and the sign word of every row of A), the gathered
+// FP32 sketch and the sizes it is for
 lsq_status lsq_sjlt_hash_launch(lsq_ctx* ctx, int64_t n, int m, int s, uint64_t seed, uint32_t t, int64_t grow0,
                                 int32_t* h, uint32_t* signs);
 lsq_status lsq_sjlt_f32(lsq_ctx* ctx, const lsq_matrix* A, int m, int s, uint64_t seed, uint32_t t, double* SA,
                         int64_t grow0);
+bool lsq_sjlt_gathers(int64_t n, int d, int m, int s);
 
 namespace {
 
@@ -1021,10 +1022,10 @@ __global__ void __launch_bounds__(SF_T, 2) srht_fix_kernel(const TA* __restrict_
 }
 
 // ------------------------------------------------------------------------------------
-// SJLT in FP64 arithmetic: s distinct rows per column of S (the hash pass of sjlt.cu), then a
-// shared-memory scatter of each data row into its s target rows.
+// SJLT in FP64 arithmetic, and in FP32 where the gather of sjlt.cu is the slower one: s distinct rows per
+// column of S (the hash pass of sjlt.cu), then a shared-memory scatter of each data row into its s target rows.
 // ------------------------------------------------------------------------------------
-// The CTA owns a tile of DC columns (4 unless m forces fewer) and a range of
+// The CTA owns a tile of DC columns (4, in FP32 8, unless m forces fewer) and a range of
 // rows; each thread takes whole rows of the tile: it loads
 // the row's s positions, sign word and DC elements once and makes s * DC shared-memory
 // additions.  Lane l visits the columns rotated by l, so the 32 lanes of an atomic spread
@@ -1545,7 +1546,13 @@ static lsq_status sjlt_run(lsq_ctx* ctx, const lsq_matrix* A, int m, int s, uint
   if ((size_t)m * DC * sizeof(TC) > budget) return LSQ_ERR_ARG;
   const int tiles = lsq_ceil_div(d, DC);
   int64_t groups = std::max<int64_t>(1, (8 * (int64_t)ctx->sm_count + tiles - 1) / tiles);
-  groups = std::min<int64_t>(groups, (n + 2047) / 2048);
+  int64_t most = (n + 2047) / 2048;
+  if (sizeof(TC) == 4) {
+    // groups of fewer rows (512 at least, chains of 4 additions) where those leave SMs idle
+    const int64_t least = std::max<int64_t>(512, std::min<int64_t>(2048, 4 * (int64_t)m / s));
+    most = std::max(most, std::min((n + least - 1) / least, (2 * (int64_t)ctx->sm_count + tiles - 1) / tiles));
+  }
+  groups = std::min(groups, most);
   const int64_t cap = std::max<int64_t>(1, ((int64_t)256 << 20) / ((int64_t)m * d * (int64_t)sizeof(TC)));
   groups = std::max<int64_t>(1, std::min(groups, cap));
   const int64_t rows_per_group = (n + groups - 1) / groups;
@@ -1561,7 +1568,9 @@ static lsq_status sjlt_run(lsq_ctx* ctx, const lsq_matrix* A, int m, int s, uint
   st = lsq_sjlt_hash_launch(ctx, n, m, s, seed, t, grow0, h, signs);
   if (st != LSQ_OK) return st;
   switch (DC) {
-    case 8: st = sjlt_launch<TC, 8>(ctx, A, m, s, h, signs, part, (int)groups, rows_per_group); break;
+    case 8:
+      if constexpr (sizeof(TC) == 4) st = sjlt_launch<TC, 8>(ctx, A, m, s, h, signs, part, (int)groups, rows_per_group);
+      break;
     case 4: st = sjlt_launch<TC, 4>(ctx, A, m, s, h, signs, part, (int)groups, rows_per_group); break;
     case 2: st = sjlt_launch<TC, 2>(ctx, A, m, s, h, signs, part, (int)groups, rows_per_group); break;
     default: st = sjlt_launch<TC, 1>(ctx, A, m, s, h, signs, part, (int)groups, rows_per_group); break;
@@ -1662,7 +1671,8 @@ static lsq_status sketch_impl(lsq_ctx* ctx, const lsq_matrix* A, int32_t type, i
         st = lsq_sjlt_tc_run(ctx, A, (int)m, s, seed, t, SA, up ? chunk_upload : nullptr, up ? &cu : nullptr, row0);
       else
         st = f64 ? sjlt_run<double>(ctx, A, (int)m, s, seed, t, SA, row0)
-                 : lsq_sjlt_f32(ctx, A, (int)m, s, seed, t, SA, row0);
+             : lsq_sjlt_gathers(A->n, (int)A->d, (int)m, s) ? lsq_sjlt_f32(ctx, A, (int)m, s, seed, t, SA, row0)
+                                                            : sjlt_run<float>(ctx, A, (int)m, s, seed, t, SA, row0);
       break;
     default:
       return LSQ_ERR_ARG;

@@ -40,3 +40,20 @@ def test_exact_on_integers(L, ctx, n, d, m, s, dtype, pad):
     ref = np.rint(O.sketch_sjlt(A, m, s, 6, 2) * np.sqrt(s))
     assert np.array_equal(np.rint(got), ref)
     assert np.abs(got - ref).max() <= 1e-12 * max(1.0, np.abs(ref).max())
+
+
+@pytest.mark.parametrize("n,d,m,s,dtype,pad", [
+    (2049, 17, 129, 4, np.float64, 1), (16385, 33, 256, 8, np.float32, 3), (40000, 130, 1025, 16, np.float64, 0),
+    (300001, 17, 64, 32, np.float32, 0), (5000, 600, 4096, 4, np.float64, 0), (610000, 101, 9000, 16, np.float32, 0),
+    (33000, 130, 2049, 32, np.float64, 0), (1 << 19, 9, 512, 8, np.float32, 0), (70001, 20, 300, 3, np.float64, 0)])
+def test_gathered_sizes(L, ctx, n, d, m, s, dtype, pad):
+    """The sizes that are gathered, either side of one and two slices of targets and of a tile, as above."""
+    test_exact_on_integers(L, ctx, n, d, m, s, dtype, pad)
+
+
+@pytest.mark.parametrize("n,d,m,s,dtype,pad", [
+    (60000, 4, 16, 16, np.float64, 0), (100003, 12, 60, 8, np.float32, 1), (2047, 40, 2000, 1, np.float64, 0),
+    (9000, 25, 6400, 8, np.float32, 3), (60001, 9, 51200, 8, np.float64, 0)])
+def test_scattered_sizes(L, ctx, n, d, m, s, dtype, pad):
+    """Sizes whose lists would cost more than their additions, with one to four columns a tile, as above."""
+    test_exact_on_integers(L, ctx, n, d, m, s, dtype, pad)
