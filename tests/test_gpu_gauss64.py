@@ -123,3 +123,17 @@ def test_non_finite(L, ctx):
     assert np.array_equal(SA[:, 1], np.sign(z) * np.inf)
     assert np.isnan(SA[:, 2]).all()
     assert not np.isfinite(SA[:, 3]).any()
+
+
+@pytest.mark.parametrize("kind", ["even", "dominant rows"])
+def test_second_panel_of_rows(L, ctx, kind):
+    """More rows than one panel of digits holds (2^18 at d <= 64), the second one short and off a stage:
+    the bound of the columns above, sqrt(n) 2^-57 of their norm, against extended precision."""
+    n, d, m = (1 << 18) + 1013, 3, 8
+    A = np.random.default_rng(6).standard_normal((n, d))
+    if kind != "even":
+        A[[5, n - 3], [1, 2]] = 1e6
+    SA = L.lsq_sketch(ctx, to_dev(A), "gauss", m, 9, t=2).cpu().numpy()
+    ref = _entries(m, n, 9, 2) @ A.astype(np.longdouble)
+    err = np.linalg.norm((SA * np.sqrt(np.longdouble(m)) - ref).astype(float), axis=0)
+    assert np.all(err < 1e-14 * np.sqrt(m) * np.linalg.norm(A, axis=0))

@@ -1,4 +1,4 @@
-"""lsq_factor's Gram matrix from digit products, at the edges of its tiles (64 x 32), stages (16 rows)
+"""lsq_factor's Gram matrix from digit products, at the edges of its tiles (64 x 32), stages (32 rows)
 and folds (128 rows), with columns scaled over +-1e120, dominant entries and a panel of rows that
 does not end on a stage: R against numpy's Householder QR of the column-normalised SA.
 
@@ -44,6 +44,13 @@ def test_r_of_scaled_columns(L, ctx, m, d, precision):
     assert np.abs(got - ref).max() <= 2e-12 * np.sqrt((ref ** 2).sum(0)).max()
     WR = (W.cpu().numpy() * s[:, None]) @ got
     assert np.abs(WR - np.eye(d)).max() < 1e-9
+
+
+@pytest.mark.parametrize("precision", ["f64", "mixed"])
+def test_second_panel_of_rows(L, ctx, precision):
+    """More rows than one panel of digits holds (2^18 at d <= 64; 299520 with 7 digits), the second one short
+    and off a stage, as above."""
+    test_r_of_scaled_columns(L, ctx, 300101, 33, precision)
 
 
 @pytest.mark.parametrize("precision", ["f64", "mixed"])

@@ -47,6 +47,31 @@ def test_sizes(n, d, ld, dtype):
     _check(rng.standard_normal((n, d)).astype(dtype), rng.standard_normal(d), ld)
 
 
+@pytest.mark.parametrize("scaled", [False, True])
+@pytest.mark.parametrize("nk", range(3, 17))
+def test_each_dot_product(nk, scaled):
+    """The w_i themselves, at every number of 32-column chunks: the last 24 columns hold a 1 in one row each
+    and p is zero there, so that v_j = w_i.  A chunk drops less than 3 units of 2^-53 of its largest
+    |a_ij p_j| (6 digit pairs of 255 x 128 on 2^40 of 2^114, for 32 columns) and rounds once as it is added;
+    the sum of two lanes and of the odd and even chunks rounds twice more."""
+    rng = np.random.default_rng(nk)
+    n, d = 304 * 200 + 77, 32 * nk - (0 if nk % 3 == 0 else rng.integers(1, 32))
+    A, p = rng.standard_normal((n, d)), rng.standard_normal(d)
+    if scaled:
+        s = 10.0 ** rng.uniform(-60, 60, d)
+        A, p = A * s, p / s
+        A *= 10.0 ** rng.uniform(-30, 30, (n, 1))
+    rows = np.concatenate([np.arange(16), [200, 201, 402, 30007, n - 78, n - 17, n - 2, n - 1]])
+    A[:, d - 24:] = 0.0
+    A[rows, np.arange(d - 24, d)] = 1.0
+    p[d - 24:] = 0.0
+    v, _ = _run(A, p)
+    P = A[rows].astype(np.longdouble) * p.astype(np.longdouble)
+    assert np.all(np.abs(v[d - 24:] - P.sum(1)) <= (nk + 6) * 2.0 ** -53 * np.abs(P).sum(1))
+    S = np.abs(A) @ np.abs(p)
+    assert np.all(np.abs(v - A.T @ (A @ p)) <= 1e-12 * (np.abs(A).T @ S))
+
+
 def test_widest_rows():
     rng = np.random.default_rng(1)
     n = 152 * 384 + 77
