@@ -30,10 +30,10 @@
 // of 255 with the fragments in registers and rows as they lie in memory (2.3-way bank conflicts on
 // average): 5.8 -> 4.2 ms a pass over the 256 problems of a batch (n 2^12..2^18, d 32..512, k 1..16; 9.2 GB);
 // 2.3 TB/s at 4 right-hand sides of d = 512 and 1.8 at 16.  What bounds it now is issue (33 instructions
-// an element at 4 right-hand sides at 2 a clock): addresses, barriers and the fold of each stage's sums.
+// an element at 4 right-hand sides at 2 a clock): addresses, barriers and the fold of each stage's sums.  (At
+// 128 registers the kernel, the exact pass with it, spills 48 bytes.)
 #pragma once
 
-constexpr int MSTAGE = 16384 + 8 * 256;  // floats of a stage at most (its rows and their padding)
 constexpr int YP = 36;                   // floats between rows of Y (16 pairs of head and remainder)
 
 struct MmaShape {
@@ -70,23 +70,10 @@ __device__ __forceinline__ void tf32_split4(const float (&a)[4], uint32_t (&h)[4
   }
 }
 
-// mbarrier of a stage filled by one bulk copy
-__device__ __forceinline__ bool tm_wait(uint64_t* bar, uint32_t parity) {
-  for (uint32_t spins = 0; spins < (1u << 24); ++spins) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(lsq_apass::smem_u32a(bar)), "r"(parity)
-        : "memory");
-    if (ok) return true;
-  }
-  return false;
-}
-
 // One FP32 chunk, rows [r0, r1) of problem pr, for the right-hand sides jl[0 .. na), na <= 8 NT:
 // out[jl[x] dp + c] = sum_rows a_c (a . p) for c < d, out[kp dp + jl[x]] = sum_rows (a . p)^2.  `phase`:
-// the parities of the four stage barriers, kept across chunks.  Called by every thread of the CTA; false if a wait gave up (every copy started has then been waited for, bounded).
+// the parities of the four stage barriers (each fills by one bulk copy), kept across chunks.  Called by every
+// thread of the CTA; false if a wait gave up (every copy started has then been waited for, bounded).
 template <int NT>
 __device__ __forceinline__ bool tm_chunk(const BProb& pr, int64_t r0, int64_t r1, double* __restrict__ out, float* smf,
                                          const int* jl, int na, uint64_t* full, uint32_t& phase) {
@@ -201,7 +188,7 @@ __device__ __forceinline__ bool tm_chunk(const BProb& pr, int64_t r0, int64_t r1
       else if (NS == 3) asm volatile("cp.async.wait_group 1;" ::: "memory");
       else asm volatile("cp.async.wait_group 2;" ::: "memory");
     } else {
-      ok = tm_wait(full + s, (phase >> s) & 1u);
+      ok = lsq_apass::ring_wait(full + s, (phase >> s) & 1u);
       phase ^= 1u << s;
     }
     if (__syncthreads_or(!ok)) {  // stage t has landed; stage t - 1 and Y are no longer read
@@ -209,7 +196,7 @@ __device__ __forceinline__ bool tm_chunk(const BProb& pr, int64_t r0, int64_t r1
       // the copies of stages t + 1 .. t + NS - 2 are still in flight: wait for them (bounded)
       if (!ms.rows)
         for (int x = t + 1; x < min(nst, t + NS - 1); ++x) {
-          tm_wait(full + x % NS, (phase >> (x % NS)) & 1u);
+          lsq_apass::ring_wait(full + x % NS, (phase >> (x % NS)) & 1u);
           phase ^= 1u << (x % NS);
         }
       break;

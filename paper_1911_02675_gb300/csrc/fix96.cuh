@@ -1,13 +1,13 @@
 // fix96.cuh -- FP64 additions on the integer pipe: 96-bit block fixed point.
 //
 // The FP64 pipe of this part does ~1.75 additions per clock per SM, the integer pipe 64 to 114.
-// Where a sum only adds and subtracts FP64 values (the Hadamard transform, the SJLT), a block of
-// values is written as integers on one scale, added exactly, and rounded back to FP64 once:
+// Where a sum only adds and subtracts FP64 values (the Hadamard transform), a block of values is
+// written as integers on one scale, added exactly, and rounded back to FP64 once:
 //   V = M 2^(31 - (emax - e)),  x = V 2^(emax - 1106),
 // M the 53-bit mantissa and e the exponent field of x, emax the largest exponent field of the
-// block.  |V| < 2^84, so 2^11 of them add without overflow; a value loses only bits below
-// 2^-84 of the block's largest, so a sum is at least as accurate as its FP64 evaluation (whose
-// every addition rounds at 2^-53 of the partial sum).
+// block.  |V| < 2^84, so 2^11 of them add without overflow; a value loses only bits below 2^-84 of
+// the block's largest, where an FP64 evaluation rounds at 2^-53 of every partial sum that the largest
+// element is in.
 #pragma once
 
 #include <stdint.h>

@@ -845,7 +845,8 @@ __global__ void __launch_bounds__(SRHT_THREADS, 1) srht_tma_kernel(
 // the other computes.  Columns with infinities or NaNs transform the signs of their infinities
 // instead: an output is +-inf where all of them agree, else NaN, as in floating point.
 // Measured (2^20 x 512 FP64, m = 1024, the whole sketch): 17.8 ms before, 4.36 ms; 144 instructions
-// an element, the integer pipe 55% busy, the rest waits on loads and shared memory.
+// an element, the integer pipe 55% busy, the rest waits on loads and shared memory.  Two CTAs an SM leave 128
+// registers: FP64 A at 4 and 8 sampled rows a thread spills 108 and 400 bytes, FP32 A at 8 256.
 constexpr int SF_T = 256, SF_DC = 4, SF_LOGN2 = 11, SF_N2 = 1 << SF_LOGN2;
 constexpr int SF_PLANE = (SF_N2 + SF_N2 / 16) * SF_DC;  // words of a plane (zphys layout)
 constexpr size_t SF_SMEM = (size_t)3 * SF_PLANE * 4;
