@@ -204,8 +204,8 @@ LSQ_API lsq_status lsq_upload_sketch(lsq_ctx* ctx, const void* host_A, int64_t h
  * paragraph; Section 6, which allows either a QR of SA or a Cholesky factor of H_S).
  *   SA : device, m x d FP64 (row-major), m >= d.
  *   R  : device, d x d FP64 output: upper triangular, positive diagonal, R^T R = H_S
- *        (Gram from exact digit products, rounded once to FP64, then Cholesky); the
- *        strict lower triangle is written as 0.
+ *        (Gram with the errors of FP64 multiply-adds or smaller, see lsq_factor_ex, then
+ *        Cholesky); the strict lower triangle is written as 0.
  *   W  : device, d x d FP64 output: W = R^{-1} (upper triangular), which lsq_solve
  *        uses to apply H_S^{-1} r = W (W^T r) as two parallel triangular products.
  * Status LSQ_ERR_RANK (after a synchronisation) if a pivot is not positive. This call
@@ -234,12 +234,15 @@ LSQ_API lsq_status lsq_factor_qr(lsq_ctx* ctx, const double* SA, int64_t m, int6
                                  double* W, int32_t* perm, int64_t* rank_out);
 
 /* lsq_factor_ex: lsq_factor with the arithmetic of the Gram matrix chosen.
- *   gram_precision : LSQ_PREC_F64 (= lsq_factor) or LSQ_PREC_MIXED.  Either way H_S is summed from
- *                    exact products of 8-bit digits of SA (columns in fixed point on the scale of their
- *                    largest element): 8 digits and 63 bits under LSQ_PREC_F64, nearer to H_S than FP64
- *                    multiply-adds; 7 digits and an error near 2^-49 of the columns' norms under
- *                    LSQ_PREC_MIXED, far below what an FP32 sketch (LSQ_SKETCH_F32) already carries.  The
- *                    Cholesky factor and the inverse stay FP64.
+ *   gram_precision : LSQ_PREC_F64 (= lsq_factor) or LSQ_PREC_MIXED, which asks for no more than the
+ *                    45 significant bits of double-FP32 elements (a relative error near 1e-13 per entry,
+ *                    far below what an FP32 sketch (LSQ_SKETCH_F32) already carries).  Columns of SA of
+ *                    which more than 5/8 of the elements lie within 2^5 of the largest, as those of a
+ *                    sketch do, are summed from exact products of 8-bit digits (fixed point on the scale
+ *                    of the largest element; 8 digits under LSQ_PREC_F64, 7 under LSQ_PREC_MIXED), with
+ *                    errors below 2^-57 and 2^-49 of the columns' norms and no larger than those of the
+ *                    sums below; the entries of other columns are summed by FP64 multiply-adds, or
+ *                    double-FP32 ones under LSQ_PREC_MIXED.  The Cholesky factor and the inverse stay FP64.
  * Other arguments, results and status as lsq_factor; LSQ_ERR_ARG for another precision. */
 LSQ_API lsq_status lsq_factor_ex(lsq_ctx* ctx, const double* SA, int64_t m, int64_t d, double* R, double* W,
                                  int32_t gram_precision);

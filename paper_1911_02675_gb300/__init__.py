@@ -285,8 +285,8 @@ def lsq_upload_sketch(ctx: Context, A_host: torch.Tensor, A: torch.Tensor, kind:
 
 def lsq_factor(ctx: Context, SA: torch.Tensor, R: torch.Tensor | None = None, W: torch.Tensor | None = None,
                precision: str = "f64"):
-    """(R, W) with R^T R = SA^T SA and W = R^{-1}; precision "mixed" forms the Gram from 7 digits
-    of SA instead of 8 (2^-49 of the columns' norms instead of 2^-57)."""
+    """(R, W) with R^T R = SA^T SA and W = R^{-1}; precision "mixed" forms the Gram to the 45 bits of
+    double-FP32 elements (7 digits of SA instead of 8, or double-FP32 sums; lsq.h)."""
     ctx.sync_stream()
     if SA.dtype != torch.float64 or not SA.is_contiguous() or not SA.is_cuda:
         raise ValueError("SA must be a contiguous CUDA float64 matrix")

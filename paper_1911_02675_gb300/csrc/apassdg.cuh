@@ -25,7 +25,7 @@
 // (whose digits do not fill their scale).
 //
 // Bound by the FP64 pipe, now with one multiply-add an element and two instructions per 32 columns of 16
-// rows: 80% busy.  (The rest is the integer work of the digits, about 25 instructions an element, and
+// rows: 70% busy by its counter.  (The rest is the integer work of the digits, about 25 instructions an element, and
 // loads of 8 rows each, whose 8 cache lines take as many cycles: chunks of 64 columns, looked at twice,
 // spent more there than they saved in FP64.  More warps or rows prefetched into L2 gave nothing.)
 // Measured: 600011 x 333, FP64 sums 859 us, chunks of 64 columns 661, this 605; 1200011 x 160, 540 us.

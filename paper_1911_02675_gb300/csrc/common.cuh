@@ -92,7 +92,7 @@ lsq_status lsq_gauss64_run(lsq_ctx* ctx, const lsq_matrix* A, int m, uint64_t se
 
 // The Gram matrix of a sketch (gram.cu): tiles (a, b) of the upper triangle, row panels and splits,
 // digits per element; lsq_gram_run adds up part[split][dp][dp] (the tiles that meet the upper triangle)
-// from the device copy of `tiles`, mag (mag_words) and planes (plane_bytes).
+// from the device copy of `tiles`, mag (mag_words, zeroed) and planes (plane_bytes).
 struct LsqGramPlan {
   int dp, dq, ns, panel, splits, rows_per_split;
   size_t plane_bytes, mag_words;

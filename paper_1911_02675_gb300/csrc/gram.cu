@@ -21,7 +21,8 @@
 //
 // Bound by the MMAs, NS (NS + 1) / 2 for each 16 x 8 x 16 product, and the latency of a stage.  Measured
 // (maximum, digits and product; before: FP64 or double-FP32 multiply-adds in tiles of 64 x 64):
-// 4096 x 1024 mixed 1100 -> 568 us, 1204 x 301 FP64 169 -> 49 us, 256 x 64 FP64 75 -> 19 us.
+// 4096 x 1024 mixed 1100 -> 568 us, 1204 x 301 FP64 169 -> 49 us, 256 x 64 FP64 75 -> 19 us; the counts cost
+// 2 us a Gram.
 #include <algorithm>
 
 #include "apass.cuh"
@@ -120,16 +121,46 @@ __device__ __noinline__ void direct_tile(const double* __restrict__ SA, int d, i
     }
 }
 
+// whether a column of the tile at (a0, b0) is left to direct_tile, given the digit kernel's counts over
+// `live` rows (columns of zeros are exact either way, those with infinities or NaNs end as NaN); each
+// thread looks at one column
+__device__ __forceinline__ bool uneven_column(const uint32_t* mag, const uint32_t* large, int live, int a0, int b0,
+                                              int d) {
+  const int tid = threadIdx.x, c = tid < BA ? a0 + tid : b0 + tid - BA;
+  if (tid >= BA + BB || c >= d) return false;
+  const uint32_t m = mag[c];
+  return m != 0u && m < 0x7FF00000u && 8ull * large[c] <= 5ull * (unsigned)live;
+}
+
+// the tiles that gram_mma_kernel leaves to it, on the same grid: at three CTAs an SM, where the product
+// kernel's registers allow one
+template <bool DF>
+__global__ void __launch_bounds__(GT, 3) gram_direct_kernel(int rows, int dp, int rows_per_split,
+                                                            const int2* __restrict__ tiles,
+                                                            const uint32_t* __restrict__ mag,
+                                                            const uint32_t* __restrict__ large,
+                                                            const double* __restrict__ SA, int row0, int live, int d,
+                                                            int accumulate, double* __restrict__ part) {
+  __shared__ __align__(16) double sm[TK * (BA + BB)];
+  const int2 tl = tiles[blockIdx.x];
+  const int a0 = tl.x * BA, b0 = tl.y * BB;
+  if (!__syncthreads_or(uneven_column(mag, large, live, a0, b0, d))) return;
+  const int k0 = blockIdx.y * rows_per_split, k1 = min(rows, k0 + rows_per_split);
+  direct_tile<DF>(SA, d, dp, row0 + min(k0, live), row0 + min(k1, live), a0, b0, mag, sm, accumulate,
+                  part + (int64_t)blockIdx.y * dp * dp);
+}
+
 // part[split][a][b] (+)= the sum over the split's rows of the panel, for one tile of H_S that meets its
 // upper triangle; planes as digits_kernel writes them for the panel's `rows` (a multiple of KC, `live` of
-// them in SA, the first one row row0), with its counts `large`
+// them in SA, the first one row row0), with its counts `large`.  direct: tiles with an uneven column are
+// summed here, too, else left to gram_direct_kernel.
 template <int NS>
 __global__ void __launch_bounds__(GT, 1) gram_mma_kernel(const uint16_t* __restrict__ planes, int rows, int dq, int dp,
                                                          int rows_per_split, const int2* __restrict__ tiles,
                                                          const uint32_t* __restrict__ mag,
                                                          const uint32_t* __restrict__ large,
                                                          const double* __restrict__ SA, int row0, int live, int d,
-                                                         int accumulate, double* __restrict__ part) {
+                                                         int accumulate, int direct, double* __restrict__ part) {
   extern __shared__ __align__(16) uint16_t sm[];  // two stages of [NS][KC][PA] and [NS][KC][PB]
   constexpr int SA_E = NS * KC * PA, SB_E = NS * KC * PB, ST = SA_E + SB_E;
   const int2 tl = tiles[blockIdx.x];
@@ -186,17 +217,9 @@ __global__ void __launch_bounds__(GT, 1) gram_mma_kernel(const uint16_t* __restr
   const int br = (lane & 7) + ((lane >> 3) & 1) * 8, bc = ((lane >> 4) & 1) * 8;    // B: (k, n) 00 10 01 11
   if (k0 < k1) load(k0, 0);  // (a short last panel leaves splits empty)
   asm volatile("cp.async.commit_group;" ::: "memory");
-  bool uneven = false;  // (columns of zeros are exact either way, those with infinities or NaNs end as NaN)
-  if (tid < BA + BB) {
-    const int c = tid < BA ? a0 + tid : b0 + tid - BA;
-    if (c < d) {
-      const uint32_t m = mag[c];
-      uneven = m != 0u && m < 0x7FF00000u && 8ull * large[c] <= 5ull * (unsigned)live;
-    }
-  }
-  if (__syncthreads_or(uneven)) {
+  if (__syncthreads_or(uneven_column(mag, large, live, a0, b0, d))) {
     asm volatile("cp.async.wait_group 0;" ::: "memory");  // (direct_tile starts with a barrier)
-    direct_tile<NS < 8>(SA, d, dp, row0 + min(k0, live), row0 + min(k1, live), a0, b0, mag, sm, accumulate,
+    if (direct) direct_tile<NS < 8>(SA, d, dp, row0 + min(k0, live), row0 + min(k1, live), a0, b0, mag, sm, accumulate,
                         out);
     return;
   }
@@ -253,6 +276,10 @@ lsq_status run(lsq_ctx* ctx, const double* SA, int m, int d, int dp, int dq, int
                const int2* d_tiles, int ntiles, uint32_t* mag, uint32_t* planes, double* part) {
   cudaStream_t s = ctx->stream;
   uint32_t* large = mag + d;  // of each panel
+  // a launch for the uneven tiles, most often empty, is worth its 2 us where tiles are many (factor of 4096 x
+  // 1024 with all columns uneven, in the product kernel and in one of their own: FP64 6.69 and 6.00 ms, mixed
+  // 3.77 and 3.21; 6.23 and 3.19 without digits)
+  const bool direct = dp <= 256;
   constexpr size_t smem = (size_t)2 * (NS * KC * PA + NS * KC * PB) * 2;
   LSQ_CUDA_TRY(cudaFuncSetAttribute(gram_mma_kernel<NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   for (int r0 = 0; r0 < m; r0 += panel) {
@@ -262,8 +289,13 @@ lsq_status run(lsq_ctx* ctx, const double* SA, int m, int d, int dp, int dq, int
     LSQ_LAUNCH_CHECK();
     gram_mma_kernel<NS><<<dim3((unsigned)ntiles, (unsigned)splits), GT, smem, s>>>(
         reinterpret_cast<const uint16_t*>(planes), rows, dq, dp, rows_per_split, d_tiles, mag, large, SA, r0,
-        std::min(rows, m - r0), d, r0 > 0 ? 1 : 0, part);
+        std::min(rows, m - r0), d, r0 > 0 ? 1 : 0, direct ? 1 : 0, part);
     LSQ_LAUNCH_CHECK();
+    if (!direct) {
+      gram_direct_kernel<NS < 8><<<dim3((unsigned)ntiles, (unsigned)splits), GT, 0, s>>>(
+          rows, dp, rows_per_split, d_tiles, mag, large, SA, r0, std::min(rows, m - r0), d, r0 > 0 ? 1 : 0, part);
+      LSQ_LAUNCH_CHECK();
+    }
     large += d;
   }
   return LSQ_OK;
@@ -296,7 +328,6 @@ LsqGramPlan lsq_gram_plan(const lsq_ctx* ctx, int m, int d, bool mixed) {
 
 lsq_status lsq_gram_run(lsq_ctx* ctx, const LsqGramPlan& p, const double* SA, int m, int d, const int2* d_tiles,
                         uint32_t* mag, uint32_t* planes, double* part) {
-  LSQ_CUDA_TRY(cudaMemsetAsync(mag, 0, p.mag_words * 4, ctx->stream));
   const int cb = (d + 31) / 32;
   const int rb = std::max(1, std::min((m + 7) / 8, (4 * ctx->sm_count + cb - 1) / cb));
   column_max_kernel<double><<<dim3((unsigned)cb, (unsigned)rb), 256, 0, ctx->stream>>>(SA, m, d, d, mag);
