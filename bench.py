@@ -60,11 +60,11 @@ SECONDARY = {"fp32_4194304x1024_gauss4096_pcg": "fp64_1048576x512_srht4096_pcg"}
 #   supplied by the sketch (profiles/solve_kernel_mixed_262144x512_srht4096.md); ("f64", 512, 1)
 #   adds the solve's own narrow_copy_kernel<16> (1.554 GB, from a full capture of that kernel).
 SOLVE_TRAFFIC = {
-    "sources_sha256": "087cd550b9f9303f7f15ab8132e1f017e5b9befc536eae6e8c89f9d918b62795",
+    "sources_sha256": "b2b798c5c3c06c0e7aa4dbdb62f3692a450e8d592d86f09fd6e5a9fdff0eed12",
     "ratios": {
-        ("f32", 1024, 0): (38971788544 + 48382720) / 38654705664,
-        ("f64", 512, 2): (14553791744 + 34407936) / 14495514624,
-        ("f64", 512, 1): (1553537240 + 14553791744 + 34407936) / 16106127360,
+        ("f32", 1024, 0): (38972263936 + 48133376) / 38654705664,
+        ("f64", 512, 2): (14553673216 + 34393344) / 14495514624,
+        ("f64", 512, 1): (1553537240 + 14553673216 + 34393344) / 16106127360,
     },
 }
 
@@ -75,8 +75,8 @@ SOLVE_TRAFFIC = {
 # --warmup 1 --no-cpu --no-e2e): reads of A plus the chunk partials written, over A's bytes.  The
 # exact passes stream A through the same stages.
 BATCH_TRAFFIC = {
-    "sources_sha256": "24f75dc8026795c2dccf6d3c67aa4f6b483408194d47cf2c6680f9ac32380ad6",
-    "ratio": (2664949504 + 27429888) / 2663123140,
+    "sources_sha256": "efa6849acd05ba648202661b6018920f88900a808845515f37e73b09755282f2",
+    "ratio": (2667505664 + 25483264) / 2663123140,
 }
 
 
