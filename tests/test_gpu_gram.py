@@ -54,13 +54,14 @@ def test_second_panel_of_rows(L, ctx, precision):
 
 
 @pytest.mark.parametrize("precision", ["f64", "mixed"])
+@pytest.mark.parametrize("d", [70, 300])
 @pytest.mark.parametrize("kind", ["even", "2^10", "2^20", "2^30", "sparse", "scaled"])
-def test_entries_where_columns_peak_in_different_rows(L, ctx, kind, precision):
+def test_entries_where_columns_peak_in_different_rows(L, ctx, kind, d, precision):
     """H_S[0][b] = R[0][0] R[0][b] entry by entry, on the scale of sum_r |a_r b_r| and not of the columns'
     norms: FP64 multiply-adds err by at most m 2^-53 of it, double-FP32 ones by 2^-44 (45 bits of each
     element) and m 2^-46 (the FP32 sums of their tails), and R[0][0], R[0][b] by a few units more."""
     g = np.random.default_rng(11)
-    m, d = 1024, 70
+    m = 1024
     X = g.standard_normal((m, d))
     if kind == "sparse":
         X *= g.random((m, d)) < 0.05
